@@ -98,12 +98,17 @@ __device__ __forceinline__ double rsqrt_(double x) {
   const double e = fma(-x * y, y, 1.0);
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
-// sqrt(x) = x / sqrt(x) for x > 0, and 0 for x = 0 (where the product would be 0 * inf)
+// sqrt(x) for x > 0, and 0 for x = 0 (where the product would be 0 * inf): with g = x y and
+// e = 1 - g y the same series gives sqrt(x) = g (1 + e/2 + 3 e^2 / 8), one operation less than
+// forming 1/sqrt(x) first, and the rounding of g enters halved (e is formed from the rounded g)
 __device__ __forceinline__ double sqrt_(double x) {
-  const double r = x * rsqrt_(x);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double g = x * y;
+  const double e = fma(-g, y, 1.0);
+  const double r = fma(g * e, fma(0.375, e, 0.5), g);
   return is_zero(x) ? 0.0 : r;
 }
-
 
 // ------------------------------------------------------------------------------------------
 // Forward-mode dual number (value + one tangent) for the adjoint kernels' local Jacobians. Every
@@ -166,11 +171,9 @@ __device__ __forceinline__ Dual rsqrt_(Dual x) {
   const double r = rsqrt_(x.v);
   return Dual(r, -0.5 * x.t * r * r * r);
 }
-// sqrt(x) = x rsqrt(x) (the value of sqrt_), derivative rsqrt(x) / 2; both 0 at x = 0
+// the value of sqrt_, derivative rsqrt(x) / 2; both 0 at x = 0
 __device__ __forceinline__ Dual sqrt_(Dual x) {
-  const double q = rsqrt_(x.v);
-  const bool z = is_zero(x.v);
-  return Dual(z ? 0.0 : x.v * q, z ? 0.0 : 0.5 * q * x.t);
+  return Dual(sqrt_(x.v), is_zero(x.v) ? 0.0 : 0.5 * rsqrt_(x.v) * x.t);
 }
 
 // x / 2 exactly as the FP64 multiply by 0.5 rounds it (ties to even), on the integer pipe: one
@@ -470,24 +473,51 @@ using FaceState = FaceStateT<double>;
 template <class T> struct PhysFluxT {
   T U[5], F[5];
   T pt, e, cf2, b2;  // cf2: the square of the fast magnetosonic speed along the normal
+  T A;               // 2 rho cf2
 };
 using PhysFlux = PhysFluxT<double>;
 
-// Total pressure and the fast magnetosonic speed of Eq. (waves:fast-speed) along the normal:
-// all the wave-speed estimates need from a state.
+// Total pressure and the fast magnetosonic speed of Eq. (waves:fast-speed) along the normal, as
+// A = 2 rho c_f^2 = P + b^2 + sqrt((P + b^2)^2 - 4 P b_n^2) with P = gamma p: neither the
+// discriminant nor A needs 1/rho.
 template <class T>
-__device__ __forceinline__ void phys_speed(const FaceStateT<T>& s, T bn, double gam, PhysFluxT<T>& o) {
-  const T bn2 = bn * bn;
+__device__ __forceinline__ void phys_speed_a(const FaceStateT<T>& s, T bn2, double gam, PhysFluxT<T>& o) {
   const T b2 = fma(s.by, s.by, fma(s.bz, s.bz, bn2));
   o.b2 = b2;
-  o.pt = fma(0.5, b2, s.p);
-  // rho c_f^2 = (P + b^2 + sqrt((P + b^2)^2 - 4 P b_n^2)) / 2 with P = gamma p: the discriminant
-  // needs no 1/rho, which enters once at the end
+  o.pt = s.p + halve(b2);
   const T P = gam * s.p;
   const T Sp = P + b2;
   T disc = fma(Sp, Sp, -(times4(bn2) * P));  // 4 bn^2 exactly, on the integer pipe
   disc = pmax(disc, T(0.0));
-  o.cf2 = halve(rcp(s.rho)) * (Sp + sqrt_(disc));
+  o.A = Sp + sqrt_(disc);
+}
+// the same with the square of the speed itself
+template <class T>
+__device__ __forceinline__ void phys_speed(const FaceStateT<T>& s, T bn, double gam, PhysFluxT<T>& o) {
+  phys_speed_a(s, bn * bn, gam, o);
+  o.cf2 = halve(rcp(s.rho)) * o.A;
+}
+// Which side has the larger fast speed, decided on A_L rho_R against A_R rho_L (no quotient).
+template <class T>
+__device__ __forceinline__ bool fast_left(const FaceStateT<T>& sl, const FaceStateT<T>& sr, const PhysFluxT<T>& L,
+                                          const PhysFluxT<T>& R, bool& finite) {
+  const double tl = val(L.A) * val(sr.rho), tr = val(R.A) * val(sl.rho);
+  finite = finite_d(tl) && finite_d(tr);
+  return dbits(tl) >= dbits(tr);
+}
+// The larger of the two fast speeds, sqrt(A / (2 rho)) of that side = (A/2) / sqrt(rho A/2): one
+// reciprocal square root in the place of two reciprocals and a square root (9 FP64 instructions
+// against 14). A state that is not finite on either side gives a speed that is not a number.
+template <class T>
+__device__ __forceinline__ T fast_max(const FaceStateT<T>& sl, const FaceStateT<T>& sr, const PhysFluxT<T>& L,
+                                      const PhysFluxT<T>& R) {
+  bool fin;
+  const bool left = fast_left(sl, sr, L, R, fin);
+  const T ah = halve(left ? L.A : R.A);
+  const T x = ah * (left ? sl.rho : sr.rho);
+  const T c = vabs(ah) * rsqrt_(x);
+  if (!fin) return T(dfrom(0x7ff8000000000000LL));
+  return is_zero(x) ? T(0.0) : c;
 }
 
 // Conserved vector and ideal-MHD flux of Eq. (mhd:conservation-laws) in the face frame, with e_tot
@@ -524,51 +554,51 @@ __device__ __forceinline__ void two_state(const PhysFluxT<T>& L, const PhysFluxT
   for (int v = 0; v < 5; ++v) F[v] = fma(wl, L.F[v], fma(wr, R.F[v], -wd * (R.U[v] - L.U[v])));
 }
 
-// Star state on one side of the contact (MK05 Eqs. 43-48).
+// Star state on one side of the contact (MK05 Eqs. 43-48), its energy apart.
 template <class T> struct StarT {
-  T rs, vs, ws, bys, bzs, es;
-  T vbs;  // u* . b* of the star state (formed with es)
+  T rs, vs, ws, bys, bzs;
 };
-// (ES = false: the energy es is not formed, and ph is not read -- the other side's star state in
-// the double-star region needs only rs, vs, ws, bys, bzs)
-template <class T, bool ES = true>
-__device__ __forceinline__ void star_state(const FaceStateT<T>& q, const PhysFluxT<T>& ph, T S, T SM,
-                                           T ptS, T bn, T bn2, StarT<T>& o) {
-  const T su = S - q.u;
-  const T ssm = S - SM;
-  const T ssminv = rcp(ssm);
-  const T rsu = q.rho * su;
-  o.rs = rsu * ssminv;
-  const T dd = fma(rsu, ssm, -bn2);
-  const T scale = fma(rsu, su, bn2);
-  if (!vgt(vabs(dd), 1e-12 * scale)) {  // degenerate: no tangential change across the fast wave
+__device__ __forceinline__ int expo(double x) { return (int)((unsigned long long)dbits(x) >> 52) & 0x7ff; }
+// whether the tangential state changes across the fast wave: |dd| > 1e-12 (m su + bn2), with
+// dd = m ssm - bn2. Settled on exponents for all but nearly degenerate states (m su + bn2 is below
+// 2^(1 + max(e_m + e_su + 2, e_bn2 + 1)), 1e-12 below 2^-39), without the FP64 instructions.
+__device__ __forceinline__ bool star_regular(double dd, double m, double su, double bn2) {
+  const int top = max(expo(m) + expo(su) - 1023 + 2, expo(bn2) + 1);
+  if (expo(dd) >= top - 38) return true;
+  return vgt(vabs(dd), 1e-12 * fma(m, su, bn2));
+}
+// m = rho su is the mass flux through the outer wave S, su = S - u, d = S_M - u, ssm = S - S_M;
+// ssminv receives 1 / ssm
+template <class T>
+__device__ __forceinline__ void star_state(const FaceStateT<T>& q, T m, T su, T d, T ssm, T bn, T bn2, T& ssminv,
+                                           StarT<T>& o) {
+  ssminv = rcp(ssm);
+  o.rs = m * ssminv;
+  const T dd = fma(m, ssm, -bn2);
+  if (!star_regular(val(dd), val(m), val(su), val(bn2))) {  // no tangential change across the fast wave
     o.vs = q.v;
     o.ws = q.w;
     o.bys = q.by;
     o.bzs = q.bz;
   } else {
     const T ddinv = rcp(dd);
-    const T cv = bn * (SM - q.u) * ddinv;
-    const T cb = fma(rsu, su, -bn2) * ddinv;
+    const T cv = bn * d * ddinv;
+    const T cb = fma(m, su, -bn2) * ddinv;
     o.vs = fma(-q.by, cv, q.v);
     o.ws = fma(-q.bz, cv, q.w);
     o.bys = q.by * cb;
     o.bzs = q.bz * cb;
   }
-  if (!ES) return;
-  const T vb = fma(q.u, bn, fma(q.v, q.by, q.w * q.bz));
-  o.vbs = fma(SM, bn, fma(o.vs, o.bys, o.ws * o.bzs));
-  o.es = (fma(su, ph.e, -ph.pt * q.u) + fma(ptS, SM, bn * (vb - o.vbs))) * ssminv;
 }
 
 // Whether the face (x/t = 0) lies inside the rotational wave S*_side = S_M -/+ |b_n| / sqrt(rho*)
 // (MK05 Eq. 51) on the side `left` of the contact (S_M >= 0 on the left): S*_left < 0 and
-// S*_right >= 0 compared as S_M^2 rho* against b_n^2, without the square root (both sides are
+// S*_right >= 0 compared as (rho* S_M) S_M against b_n^2, without the square root (both sides are
 // non-negative, so the bit patterns order them). The reverse sweep takes the same decision.
 template <class T>
 __device__ __forceinline__ bool hlld_in_rotational(bool left, T SM, T rs, T bn2) {
   const double sm = val(SM);
-  const long long q = dbits(sm * sm * val(rs)), b = dbits(val(bn2));
+  const long long q = dbits(val(rs) * sm * sm), b = dbits(val(bn2));
   return left ? q < b : q <= b;
 }
 
@@ -589,80 +619,96 @@ __device__ __forceinline__ FaceStateT<T> pick(bool left, const FaceStateT<T>& a,
 // the flux is that side's physical flux; inside it the face x/t = 0 lies on the side of the
 // contact given by sgn(S_M), and only that side's star state is formed, and the other side's star
 // state and the double-star state (MK05 Eqs. 49-63) only when the face lies inside that side's
-// rotational wave. Same values as forming all four states and selecting. The side is chosen before
-// the one physical flux vector a face needs is formed, so that the lanes of a warp on either side
-// of the fan or inside it form it together.
+// rotational wave.
+// The Rankine-Hugoniot relations behind the star states make every one of their fluxes
+// (F + S (U* - U), and F* + S* (U** - U*)) the physical flux of the state at x/t = 0, with S_M for
+// its normal velocity and p_t* for its total pressure. So the branches only form that state
+// (density, tangential velocity and field, energy, u . b), and one flux is formed at the end by all
+// lanes of a warp together: in the fan 105 FP64 instructions a face against 143 when the flux
+// vectors were differenced across the waves, and 154 against 218 in the double-star region
+// (counted on the formulas; with fast_max and sqrt_ the 256^3 turbulence step took 46.9 ms against
+// 49.4, the 128^3 Alfven step 8.43 against 9.64, 96 subsonic patches 19.9 against 22.8). MK05
+// Eqs. 38 and 41 are taken relative to the side's own velocity:
+// d = S_M - u = (m_o (u_R - u_L) + p_L - p_R) / (m_R - m_L) with the other side's mass flux m_o,
+// and p_t* = p_t + m d.
+// A component of the double-star state differs from the star state a of its side by
+// x = (sqrt(rho_b*) (v_b - v_a) + s (B_b - B_a)) / (sqrt(rho_a*) + sqrt(rho_b*)) in the velocity and
+// by s sqrt(rho_a*) x in the field (MK05 Eqs. 59-62, b the other side's star state, s = sgn(b_n)
+// on the left and -sgn(b_n) on the right).
 template <class T>
-__device__ __forceinline__ void hlld(const FaceStateT<T>& sl, const FaceStateT<T>& sr, T bn, double gm1inv,
+__device__ __forceinline__ void hlld(const FaceStateT<T>& sl, const FaceStateT<T>& sr, T bn, T bn2, double gm1inv,
                                      const PhysFluxT<T>& L, const PhysFluxT<T>& R, T SL, T SR, T* F) {
   const bool supL = gt0(SL);
   const bool fan = !supL && !lt0(SR);
-  T mL = 0.0, mR = 0.0, SM = 0.0, ptS = 0.0;
+  T suL = 0.0, suR = 0.0, mL = 0.0, mR = 0.0, du = 0.0, dpt = 0.0, nL = 0.0, dinv = 0.0, SM = 0.0;
   if (fan) {
-    mL = (SL - sl.u) * sl.rho;  // mass fluxes through the outer waves
-    mR = (SR - sr.u) * sr.rho;
-    const T dinv = rcp(mR - mL);
-    SM = ((mR * sr.u - mL * sl.u) + (L.pt - R.pt)) * dinv;  // MK05 Eq. 38
-    ptS = (mR * L.pt - mL * R.pt + mL * mR * (sr.u - sl.u)) * dinv;  // MK05 Eq. 41
+    suL = SL - sl.u;
+    suR = SR - sr.u;
+    mL = suL * sl.rho;  // mass fluxes through the outer waves
+    mR = suR * sr.rho;
+    dinv = rcp(mR - mL);
+    du = sr.u - sl.u;
+    dpt = L.pt - R.pt;
+    nL = fma(mR, du, dpt);
+    SM = fma(nL, dinv, sl.u);
   }
   const bool left = fan ? ge0(SM) : supL;
   const FaceStateT<T> q = pick(left, sl, sr);
-  PhysFluxT<T> P;
-  P.b2 = left ? L.b2 : R.b2;
-  P.pt = left ? L.pt : R.pt;
-  phys_flux(q, bn, gm1inv, P);
-  if (!fan) {
-    for (int v = 0; v < 5; ++v) F[v] = P.F[v];
-    return;
+  const T b2 = left ? L.b2 : R.b2;
+  T pt = left ? L.pt : R.pt;
+  // the state at x/t = 0: outside the fan the side's own
+  T rho = q.rho, un = q.u, v = q.v, w = q.w, by = q.by, bz = q.bz;
+  T e = fma(q.p, gm1inv, halve(fma(q.rho, fma(q.u, q.u, fma(q.v, q.v, q.w * q.w)), b2)));
+  T ub = fma(q.u, bn, fma(q.v, q.by, q.w * q.bz));
+  if (fan) {
+    const T su = left ? suL : suR, m = left ? mL : mR;
+    const T nS = left ? nL : fma(mL, du, dpt);
+    const T d = nS * dinv;  // S_M - u of the side
+    const T ptS = fma(m, d, pt);
+    const T ssm = su - d;
+    T ssminv;
+    StarT<T> a;
+    star_state(q, m, su, d, ssm, bn, bn2, ssminv, a);
+    const T vbs = fma(SM, bn, fma(a.vs, a.bys, a.ws * a.bzs));
+    const T es = fma(bn, ub - vbs, fma(ptS, SM, fma(su, e, -(pt * q.u)))) * ssminv;
+    rho = a.rs;
+    un = SM;
+    pt = ptS;
+    v = a.vs;
+    w = a.ws;
+    by = a.bys;
+    bz = a.bzs;
+    e = es;
+    ub = vbs;
+    if (hlld_in_rotational(left, SM, a.rs, bn2)) {
+      // the other side's star state (its density, tangential velocity and field)
+      const FaceStateT<T> qo = pick(!left, sl, sr);
+      const T suo = left ? suR : suL, mo = left ? mR : mL;
+      const T ssmo = suo - (SM - qo.u);
+      T oinv;
+      StarT<T> o;
+      star_state(qo, mo, suo, SM - qo.u, ssmo, bn, bn2, oinv, o);
+      const T sq = sqrt_(a.rs), sqo = sqrt_(o.rs);
+      const T inv = rcp(sq + sqo);
+      // b_n != 0 here (with b_n = 0 there is no rotational wave), so s = +-1 is a sign flip
+      const bool neg = lt0(bn) == left;
+      const T xv = fma(sqo, o.vs - a.vs, neg_if(neg, o.bys - a.bys)) * inv;
+      const T xw = fma(sqo, o.ws - a.ws, neg_if(neg, o.bzs - a.bzs)) * inv;
+      const T ssq = neg_if(neg, sq);
+      v = a.vs + xv;
+      w = a.ws + xw;
+      by = fma(ssq, xv, a.bys);
+      bz = fma(ssq, xw, a.bzs);
+      ub = fma(SM, bn, fma(v, by, w * bz));
+      e = fma(ssq, ub - vbs, es);
+    }
   }
-  const T bn2 = bn * bn;
-  const T abn = vabs(bn);
-  const T S = left ? SL : SR;
-  StarT<T> a;
-  star_state(q, P, S, SM, ptS, bn, bn2, a);
-  const T Usa[5] = {a.rs, a.rs * SM, a.rs * a.vs, a.rs * a.ws, a.es};
-  T Fs[5];
-#pragma unroll
-  for (int v = 0; v < 5; ++v) Fs[v] = fma(S, Usa[v] - P.U[v], P.F[v]);
-  if (!hlld_in_rotational(left, SM, a.rs, bn2)) {
-    for (int v = 0; v < 5; ++v) F[v] = Fs[v];
-    return;
-  }
-  const T isqa = rsqrt_(a.rs);
-  const T Ss = left ? SM - abn * isqa : SM + abn * isqa;  // MK05 Eq. 51
-  // inside the rotational wave of this side: the other side's star state (its density, velocity
-  // and field only) and the double star
-  const FaceStateT<T> qo = pick(!left, sl, sr);
-  StarT<T> b;
-  star_state<T, false>(qo, P, left ? SR : SL, SM, ptS, bn, bn2, b);
-  const T isqb = rsqrt_(b.rs);
-  const T rsL = left ? a.rs : b.rs, rsR = left ? b.rs : a.rs;
-  const T vsL = left ? a.vs : b.vs, vsR = left ? b.vs : a.vs;
-  const T wsL = left ? a.ws : b.ws, wsR = left ? b.ws : a.ws;
-  const T bysL = left ? a.bys : b.bys, bysR = left ? b.bys : a.bys;
-  const T bzsL = left ? a.bzs : b.bzs, bzsR = left ? b.bzs : a.bzs;
-  const T iL = left ? isqa : isqb, iR = left ? isqb : isqa;
-  const T sqL = rsL * iL, sqR = rsR * iR;
-  // sgn(b_n) is +-1 here (the double-star branch needs b_n != 0: with b_n = 0, S*_side = S_M),
-  // so the products by it are sign flips
-  const bool nb = lt0(bn);
-  const T inv = rcp(sqL + sqR);
-  const T vss = fma(sqL, vsL, fma(sqR, vsR, neg_if(nb, bysR - bysL))) * inv;
-  const T wss = fma(sqL, wsL, fma(sqR, wsR, neg_if(nb, bzsR - bzsL))) * inv;
-  const T sLR = sqL * sqR;
-  const T byss = fma(sqL, bysR, fma(sqR, bysL, neg_if(nb, sLR * (vsR - vsL)))) * inv;
-  const T bzss = fma(sqL, bzsR, fma(sqR, bzsL, neg_if(nb, sLR * (wsR - wsL)))) * inv;
-  const T vbss = fma(SM, bn, fma(vss, byss, wss * bzss));
-  const T sq = left ? sqL : sqR;
-  const T vbs = a.vbs;
-  T Uss[5];
-  Uss[0] = a.rs;
-  Uss[1] = a.rs * SM;
-  Uss[2] = a.rs * vss;
-  Uss[3] = a.rs * wss;
-  Uss[4] = fma(neg_if(left != nb, sq), vbs - vbss, a.es);  // (-1 on the left) sq (vbs - vbss) sgn(b_n)
-#pragma unroll
-  for (int v = 0; v < 5; ++v) F[v] = fma(Ss, Uss[v] - Usa[v], Fs[v]);
+  const T mu = rho * un;
+  F[0] = mu;
+  F[1] = fma(mu, un, pt - bn2);
+  F[2] = fma(mu, v, -(bn * by));
+  F[3] = fma(mu, w, -(bn * bz));
+  F[4] = fma(e + pt, un, -(ub * bn));
 }
 
 // Full face solve: flux of {rho, m_n, m_t1, m_t2, e}, alpha+/-, and the Q26 face velocity.
@@ -671,27 +717,31 @@ __device__ __forceinline__ void riemann(const FaceStateT<T>& sl, const FaceState
                                         double gam, double gm1inv, T* F, T& ap,
                                         T& am, T& ustar) {
   PhysFluxT<T> L, R;
-  phys_speed(sl, bn, gam, L);
-  phys_speed(sr, bn, gam, R);
+  const T bn2 = bn * bn;
   T SL = 0.0, SR = 0.0;
   if (RS == RS_LLF) {
+    phys_speed(sl, bn, gam, L);
+    phys_speed(sr, bn, gam, R);
     const T a = pmax(vabs(sl.u) + sqrt_(L.cf2), vabs(sr.u) + sqrt_(R.cf2));
     ap = a;
     am = a;
   } else {
+    phys_speed_a(sl, bn2, gam, L);
+    phys_speed_a(sr, bn2, gam, R);
     // Eq. (alpha-pm) = MK05 Eq. 67 speeds
-    const T cmax = sqrt_(pmax(L.cf2, R.cf2));  // = max of the two speeds, one square root
+    const T cmax = fast_max(sl, sr, L, R);
     const T umax = vmax(sl.u, sr.u), umin = vmin(sl.u, sr.u);
     SR = umax + cmax;
     SL = umin - cmax;
     ap = vmax(0.0, SR);
-    am = vmax(0.0, cmax - umin);
+    // max(0, -SL), a speed that is not a number kept: -SL is cmax - umin, without forming it
+    am = (unsigned long long)dbits(val(SL)) <= 0x7ff0000000000000ULL ? T(0.0) : neg_if(dbits(val(SL)) < 0, SL);
   }
   const T sum = ap + am;
   const bool zero = is_zero(sum);
   const T inv = zero ? 0.0 : rcp(sum);
   if (RS == RS_HLLD) {
-    hlld(sl, sr, bn, gm1inv, L, R, SL, SR, F);  // (reads L, R's pt and b2 only)
+    hlld(sl, sr, bn, bn2, gm1inv, L, R, SL, SR, F);  // (reads L, R's pt and b2 only)
   } else {
     phys_flux(sl, bn, gm1inv, L);
     phys_flux(sr, bn, gm1inv, R);
