@@ -302,7 +302,7 @@ mhd_status mhd_batch_set_schedule(mhd_batch *batch, int seg, int order, int bloc
 mhd_status mhd_batch_set_launches(mhd_batch *batch, int launches_per_stage);
 
 /* Autotuner: times one step for every candidate schedule (1 or 3 launches per stage; seg in
- * {16, 32, 64, 128}; both orders; 1 .. max CTAs per SM of the first launch) on a scratch copy of
+ * {16, 32, 64, 128}; both orders; as many CTAs per SM of the first launch as fit, or one fewer) on a scratch copy of
  * `state` (left unchanged; the copy is allocated and freed here), keeps the fastest and returns
  * it (any output pointer may be NULL). The choice is remembered for the process, keyed by the
  * device, the scheme, whether eta is zero and the histogram of patch sizes: a later call with the

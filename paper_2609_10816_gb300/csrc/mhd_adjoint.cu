@@ -76,11 +76,12 @@ __device__ __forceinline__ void recon_jac(const double* q, double* JL, double* J
     // the decisions of Rec<REC_PPM_EP> on the same window
     const double e0 = q[1] - q[0], e1 = q[2] - q[1], e2 = q[3] - q[2], e3 = q[4] - q[3];
     const int s0 = sgn_code(e0), s1 = sgn_code(e1), s2 = sgn_code(e2), s3 = sgn_code(e3);
-    const int ka = sgn_code(e1 - e0), kb = sgn_code(e2 - e1), kc = sgn_code(e3 - e2);
+    const int ka = cmp_code(e1, e0), kb = cmp_code(e2, e1), kc = cmp_code(e3, e2);
     const bool xa = ext_code(s0, s1, s2), xb = ext_code(s1, s2, s3);
     int pa, pb;  // 0: fourth-order value, 1: the lower cell's value, 2: the upper cell's
-    const double aL = ppm_ep_face(q[0], q[1], q[2], q[3], xa && same_code(ka, kb), pa);
-    const double aR = ppm_ep_face(q[1], q[2], q[3], q[4], xb && same_code(kb, kc), pb);
+    double ra, sa, rb, sb;
+    ppm_ep_face(q[1], q[2], e0, e1, e2, xa && same_code(ka, kb), pa, ra, sa);
+    ppm_ep_face(q[2], q[3], e1, e2, e3, xb && same_code(kb, kc), pb, rb, sb);
     if (pa == 0) {
       JL[0] = -1.0 / 12.0; JL[1] = 7.0 / 12.0; JL[2] = 7.0 / 12.0; JL[3] = -1.0 / 12.0;
     } else {
@@ -92,7 +93,7 @@ __device__ __forceinline__ void recon_jac(const double* q, double* JL, double* J
       JR[pb == 1 ? 2 : 3] = 1.0;
     }
     if (!((xa || xb) && same_code(ka, kb) && same_code(kb, kc))) {
-      const int mc = ppm_mono_case(aR - q[2], q[2] - aL);
+      const int mc = ppm_mono_case(rb, sa);
       if (mc == PPM_FLAT) {
 #pragma unroll
         for (int k = 0; k < 5; ++k) JL[k] = JR[k] = 0.0;
@@ -126,9 +127,10 @@ __device__ __forceinline__ void recon_jac(const double* q, double* JL, double* J
     JL[1] += 0.5; JL[2] += 0.5;
     JR[2] += 0.5; JR[3] += 0.5;
     // monotonicity (ppm_mono on the values)
-    const double d0 = vl_slope2(e0, e1), d1 = vl_slope2(e1, e2), d2 = vl_slope2(e2, e3);
-    const double aL = ppm_iface(q[1], e1, d0, d1), aR = ppm_iface(q[2], e2, d1, d2);
-    const int mc = ppm_mono_case(aR - q[2], q[2] - aL);
+    double ra, sa, rb, sb;
+    ppm_split(e0, e1, e2, ra, sa);
+    ppm_split(e1, e2, e3, rb, sb);
+    const int mc = ppm_mono_case(rb, sa);
     if (mc == PPM_FLAT) {
 #pragma unroll
       for (int k = 0; k < 5; ++k) JL[k] = JR[k] = 0.0;
@@ -467,24 +469,22 @@ __global__ void __launch_bounds__(128) k_adj_edge_rec(AdjDev A) {
 // no atomics: each point's sum is formed by one thread.
 struct RevPPM {
   double q0, q1, q2;          // q_i, q_{i+1}, q_{i+2}
-  double e1;                  // e_{i+1}
-  double d0, d1;              // d_i, d_{i+1}
+  double e0, e1;              // e_i, e_{i+1}
   double am, bm, a0, b0, a1, b1;  // slope jacobians of d_{i-1}, d_i, d_{i+1}
-  double fL, fR;              // f_{i-1/2}, f_{i+1/2}
+  double s1, s2, sn;          // f_{i+1/2} - q_i, q_i - f_{i-1/2}, q_{i+1} - f_{i+1/2}
   double lfp, ld, le, g2, g1;  // adjoints: upper value of point i-1, d_{i-1}, e_{i-2}, q_{i-2}, q_{i-1}
 
   // v = q_{i-2} .. q_{i+2} for the first step i
   __device__ __forceinline__ void init(const double* v) {
-    const double e0 = v[1] - v[0], e1_ = v[2] - v[1], e2 = v[3] - v[2], e3 = v[4] - v[3];
-    const double dm = vl_slope2(e0, e1_);
-    vl_slope2_jac(e0, e1_, am, bm);
-    d0 = vl_slope2(e1_, e2);
+    const double em = v[1] - v[0], e1_ = v[2] - v[1], e2 = v[3] - v[2], e3 = v[4] - v[3];
+    vl_slope2_jac(em, e1_, am, bm);
     vl_slope2_jac(e1_, e2, a0, b0);
-    d1 = vl_slope2(e2, e3);
     vl_slope2_jac(e2, e3, a1, b1);
-    fL = ppm_iface(v[1], e1_, dm, d0);
-    fR = ppm_iface(v[2], e2, d0, d1);
+    double r;
+    ppm_split(em, e1_, e2, r, s2);
+    ppm_split(e1_, e2, e3, s1, sn);
     q0 = v[2]; q1 = v[3]; q2 = v[4];
+    e0 = e2;
     e1 = e3;
     lfp = ld = le = g2 = g1 = 0.0;
   }
@@ -492,7 +492,7 @@ struct RevPPM {
   // q_{i-2}.
   __device__ __forceinline__ double step(double lam_lo, double lam_hi, double qn) {
     double lL = lam_lo, lR = lam_hi, gi = 0.0;
-    const int mc = ppm_mono_case(fR - q0, q0 - fL);
+    const int mc = ppm_mono_case(s1, s2);
     if (mc == PPM_FLAT) {  // aL = aR = q_i
       gi = lam_lo + lam_hi;
       lL = lR = 0.0;
@@ -517,15 +517,14 @@ struct RevPPM {
     g2 = g1; g1 = gi; le = le1; ld = ldi; lfp = lR;
     // forward values of the next step
     const double en = qn - q2;            // e_{i+2}
-    const double dn = vl_slope2(e1, en);  // d_{i+2}
     double an, bn;
     vl_slope2_jac(e1, en, an, bn);
-    const double fn = ppm_iface(q1, e1, d1, dn);  // f_{i+3/2}
+    s2 = sn;
+    ppm_split(e0, e1, en, s1, sn);        // f_{i+3/2}
     am = a0; bm = b0; a0 = a1; b0 = b1; a1 = an; b1 = bn;
-    d0 = d1; d1 = dn;
+    e0 = e1;
     e1 = en;
     q0 = q1; q1 = q2; q2 = qn;
-    fL = fR; fR = fn;
     return out;
   }
 };

@@ -142,7 +142,7 @@ void run_stage(mhd_ctx* c, const mhd::Dev& D, const Decoded& sc, PrimSource prim
 
 void mhd::set_call_error(const char* msg) { g_create_err = msg; }
 
-int mhd::resident_blocks(const void* fn, int threads) {
+int mhd::resident_blocks(const void* fn, int threads, int smem) {
   static std::mutex mu;
   static std::map<std::tuple<const void*, int, int>, int> cache;
   int dev = 0;
@@ -152,7 +152,8 @@ int mhd::resident_blocks(const void* fn, int threads) {
   auto it = cache.find(key);
   if (it != cache.end()) return it->second;
   int per_sm = 0, nsm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, 0) != cudaSuccess || per_sm < 1)
+  if (smem > 0) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, (size_t)smem) != cudaSuccess || per_sm < 1)
     per_sm = 1;
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) nsm = 1;
   cache[key] = per_sm * nsm;

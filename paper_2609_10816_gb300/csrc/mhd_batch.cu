@@ -114,6 +114,23 @@ static StageKernel batch_kernel_of(int recon, int which, int rs, int emf) {
 }
 // the first launch of a stage: the one launch per stage (one) or the face launch of three
 static StageKernel stage_kernel(int recon, int rs, bool one) { return batch_kernel_of(recon, one ? 0 : 1, rs, 0); }
+// dynamic shared memory of a block of the stage's first launch (the face sweep's windows)
+static int stage_smem(int recon) {
+  switch (recon) {
+    case REC_PC: return face_smem_bytes<REC_PC>();
+    case REC_PLM_MC: return face_smem_bytes<REC_PLM_MC>();
+    case REC_PLM_MINMOD: return face_smem_bytes<REC_PLM_MINMOD>();
+    case REC_PPM: return face_smem_bytes<REC_PPM>();
+    default: return face_smem_bytes<REC_PPM_EP>();
+  }
+}
+// CTAs per SM of the stage's first launch that fit, with the kernel allowed its shared memory
+static cudaError_t stage_occupancy(int recon, int rs, bool one, int* per_sm) {
+  const void* k = (const void*)stage_kernel(recon, rs, one);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, stage_smem(recon));
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k, kFaceThreads, (size_t)stage_smem(recon));
+}
 // the second launch of three (edge, update and flag phases)
 static StageKernel rest_kernel(int recon, int emf) { return batch_kernel_of(recon, 2, 0, emf); }
 
@@ -329,7 +346,7 @@ mhd_status enqueue_step(mhd_batch* b, const mhd_batch_state* s, double cfl, int 
   mhd::StageKernel kf = mhd::stage_kernel(recon, rs, one), kr = mhd::rest_kernel(recon, emf);
   int per_sm = 0, per_sm_rest = 0;
   int per_sm_fofc = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, 128, 0);
+  cudaError_t e = mhd::stage_occupancy(recon, rs, one, &per_sm);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_rest, kr, 128, 0);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_fofc, (const void*)mhd::k_batch_fofc, 128, 0);
@@ -357,6 +374,7 @@ mhd_status enqueue_step(mhd_batch* b, const mhd_batch_state* s, double cfl, int 
       std::memset(&lc, 0, sizeof(lc));
       lc.gridDim = dim3(part == 1 ? grid_rest : (part == 0 ? grid_face : grid_fofc));
       lc.blockDim = dim3(128);
+      lc.dynamicSmemBytes = part == 0 ? (size_t)mhd::stage_smem(recon) : 0;
       lc.stream = st;
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeCooperative;
@@ -654,10 +672,8 @@ mhd_status mhd_batch_tune(mhd_batch* b, const mhd_batch_state* s, double cfl, in
   if (e != cudaSuccess) return bcuda(b, e, "cudaMalloc");
   mhd_batch_state t = {cpy, cpy + 5 * b->ncell};
   int per_sm[2] = {0, 0};  // CTAs per SM of the first launch: one launch per stage, three
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], mhd::stage_kernel(scheme & 0xf, (scheme >> 4) & 0xf, true),
-                                                128, 0);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], mhd::stage_kernel(scheme & 0xf, (scheme >> 4) & 0xf, false),
-                                                128, 0);
+  mhd::stage_occupancy(scheme & 0xf, (scheme >> 4) & 0xf, true, &per_sm[0]);
+  mhd::stage_occupancy(scheme & 0xf, (scheme >> 4) & 0xf, false, &per_sm[1]);
   const int segs[] = {16, 32, 64, 128};
   float best = 1e30f;
   int bs = 64, bo = 1, bb = 0, bl = 3;
@@ -669,7 +685,7 @@ mhd_status mhd_batch_tune(mhd_batch* b, const mhd_batch_state* s, double cfl, in
   for (int form = 0; form < 2 && st == MHD_OK; ++form)
   for (int seg : segs)
     for (int order = 0; order < 2 && st == MHD_OK; ++order)
-      for (int bps = 1; bps <= std::max(1, per_sm[form]) && st == MHD_OK; ++bps) {
+      for (int bps = std::max(1, per_sm[form] - 1); bps <= std::max(1, per_sm[form]) && st == MHD_OK; ++bps) {
         st = mhd_batch_set_schedule(b, seg, order, bps, 0);
         if (st == MHD_OK) st = mhd_batch_set_launches(b, form == 0 ? 1 : 3);
         if (st != MHD_OK) break;

@@ -134,6 +134,8 @@ constexpr int kRestIlp = 2;
 // CTAs of 128 threads per SM that the second launch of a stage is compiled to fit (one fewer for
 // FS18, whose bottom/top sweep carries five reconstruction windows)
 constexpr int kRestMinBlocks = 4;
+// and the one launch per stage (which holds every EMF scheme's phases)
+constexpr int kStageMinBlocks = 3;
 
 // The phases of a stage, as device functions that the stage's launches run: false when a grid
 // barrier gave up (the block then leaves the kernel).
@@ -341,7 +343,7 @@ __device__ __forceinline__ void stage_all(const BatchDev& B) {
   fofc_part(B);
 }
 template <int RC, int RS>
-__global__ void __launch_bounds__(128) k_batch_stage(BatchDev B) {
+__global__ void __launch_bounds__(kFaceThreads, kStageMinBlocks) k_batch_stage(BatchDev B) {
   switch (B.emf) {  // uniform over the grid
     case EMF_FS18: stage_all<RC, RS, EMF_FS18>(B); break;
     case EMF_B25A: stage_all<RC, RS, EMF_B25A>(B); break;
@@ -349,7 +351,7 @@ __global__ void __launch_bounds__(128) k_batch_stage(BatchDev B) {
   }
 }
 template <int RC, int RS>
-__global__ void __launch_bounds__(128) k_batch_face(BatchDev B) {
+__global__ void __launch_bounds__(kFaceThreads, kFaceMinBlocks) k_batch_face(BatchDev B) {
   face_part<RC, RS>(B);
 }
 template <int RC, int EMF>

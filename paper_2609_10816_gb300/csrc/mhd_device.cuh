@@ -210,12 +210,16 @@ struct Line {
 // takes the value at m + LA and returns the left/right states of the interface between
 // points m-1 and m (left = upper value of point m-1, right = lower value of point m). Every
 // point's slope, interface value and limiter run exactly once per sweep.
+// For sweeps that keep their windows in shared memory: each() visits the NS doubles of the state,
+// and code holds NB more bits.
 // ------------------------------------------------------------------------------------------
 template <int R> struct Rec;
 
 template <> struct Rec<REC_PC> {
-  static constexpr int LB = 1, LA = 0;
+  static constexpr int LB = 1, LA = 0, NS = 1, NB = 0;
   double prev;
+  int code;
+  template <class F> __device__ __forceinline__ void each(F f) { f(0, prev); }
   __device__ __forceinline__ void init(const double* q) { prev = q[0]; }
   __device__ __forceinline__ void step(double qn, double& L, double& R) {
     L = prev;
@@ -240,8 +244,14 @@ __device__ __forceinline__ T half_slope_minmod(T dl, T dr) {
 }
 
 template <int R> struct RecPLM {
-  static constexpr int LB = 2, LA = 1;
+  static constexpr int LB = 2, LA = 1, NS = 3, NB = 0;
   double qb, dl, aRprev;  // q[m], q[m] - q[m-1], upper value of point m-1
+  int code;
+  template <class F> __device__ __forceinline__ void each(F f) {
+    f(0, qb);
+    f(1, dl);
+    f(2, aRprev);
+  }
   __device__ __forceinline__ double hs(double a, double b) const {
     return R == REC_PLM_MC ? half_slope_mc(a, b) : half_slope_minmod(a, b);
   }
@@ -287,80 +297,157 @@ __device__ __forceinline__ long long twice_bits(long long b) {
 __device__ __forceinline__ double times4(double m) { return dfrom(twice_bits(twice_bits(dbits(m)))); }
 __device__ __forceinline__ Dual times4(Dual m) { return Dual(times4(m.v), 4.0 * m.t); }
 
-template <class T>
-__device__ __forceinline__ T vl_slope2(T dl, T dr) {
-  if (!same_sign(dl, dr)) return T(0.0);
-  const T s = dl + dr;
-  const T m = pmin(vabs(s), times4(pmin(vabs(dl), vabs(dr))));
+__device__ __forceinline__ double vl_slope2(double dl, double dr) {
+  if (!same_sign(dl, dr)) return 0.0;
+  const double s = dl + dr;
+  const double m = pmin(vabs(s), times4(pmin(vabs(dl), vabs(dr))));
   return with_sign(m, s);
 }
-template <class T>
-__device__ __forceinline__ T ppm_iface(T q0, T dq, T d20, T d21) {
-  return fma(-(d21 - d20), T(1.0 / 12.0), fma(T(0.5), dq, q0));
-}
 // With s1, s2 of one sign, u = s2 - 2 s1 = (a6 - da)/2 has the sign of s1 exactly when
-// |s2| > 2|s1|, and v = 2 s2 - s1 = (a6 + da)/2 the sign of -s1 exactly when 2|s2| < |s1| (u and v
-// are single roundings of exact differences of doubles, so their signs are exact): the two tests
-// compare bit patterns, and the one correction that applies is a single FMA.
+// |s2| > 2|s1|, and v = 2 s2 - s1 = (a6 + da)/2 the sign of -s1 exactly when 2|s2| < |s1|: the two
+// tests compare bit patterns (one more in the exponent is the doubling), and the one correction
+// that applies is a single FMA.
 enum { PPM_FLAT = 0, PPM_FIX_L = 1, PPM_FIX_R = 2, PPM_KEEP = 3 };
 // which constraint applies for s1 = aR - a, s2 = a - aL
 __device__ __forceinline__ int ppm_mono_case(double s1, double s2) {
-  if (!same_sign(s1, s2)) return PPM_FLAT;                        // a is an extremum
-  const long long m1 = mag_bits(s1), m2 = mag_bits(s2);
-  if (m2 > twice_bits(m1)) return PPM_FIX_L;                        // aL = 3a - 2aR = a - 2 s1
-  if (twice_bits(m2) < m1) return PPM_FIX_R;                        // aR = 3a - 2aL = a + 2 s2
+  const long long m1 = mag_bits(s1), m2 = mag_bits(s2), two = 1LL << 52;
+  if ((dbits(s1) ^ dbits(s2)) < 0 || m1 == 0 || m2 == 0) return PPM_FLAT;  // a is an extremum
+  if (m2 > m1 + two) return PPM_FIX_L;                                     // aL = 3a - 2aR = a - 2 s1
+  if (m2 + two < m1) return PPM_FIX_R;                                     // aR = 3a - 2aL = a + 2 s2
   return PPM_KEEP;
 }
-template <class T>
-__device__ __forceinline__ void ppm_mono(T a, T& aL, T& aR) {
-  const T s1 = aR - a, s2 = a - aL;
-  const int c = ppm_mono_case(val(s1), val(s2));
+__device__ __forceinline__ void ppm_mono(double a, double s1, double s2, double& aL, double& aR) {
+  const int c = ppm_mono_case(s1, s2);
   if (c == PPM_FLAT) {
     aL = a;
     aR = a;
   } else if (c != PPM_KEEP) {
     const bool l = c == PPM_FIX_L;
-    const T r = fma(l ? -2.0 : 2.0, l ? s1 : s2, a);
+    const double r = fma(l ? -2.0 : 2.0, l ? s1 : s2, a);
     if (l) aL = r; else aR = r;
   }
 }
 
+// The interface value on the integer pipe. With d = q1 - q0 across the interface and the
+// differences dl, dn on either side, the interface lies r = d/2 + (dq2_0 - dq2_1)/12 above q0 and
+// s = d - r below q1. The limited slopes never exceed 4|d| in size, so everything is a fixed-point
+// number in units of d's exponent: |d| is its 53-bit significand times 2^7 (in [2^59, 2^60)), the
+// neighbours are shifted to the same scale (differences of the other sign to 0, and those of at
+// least 2^3 |d|'s binade clamped there, where the limiter takes 4|d| whatever they are), and sums,
+// minima and the division by 12 are 64-bit integer operations. r and s lie in [|d|/6, 5|d|/6] with
+// d's sign, so each is normalised by a shift of 4 to 7 bits and rounded once (to nearest; the bits
+// shifted out and the division leave an error below a sixteenth of that rounding unit).
+// The FP64 pipe takes 64 cycles for an instruction of a warp and the integer pipe 2: per value
+// reconstructed this leaves 3 FP64 instructions (the new difference, q0 + r, and the monotonicity
+// correction) of 8, for about 60 more integer ones. The 256^3 bottom/top edge sweeps, which only
+// reconstruct, took 1.9 ms a step against 3.2, and a face 119 FP64 instructions against 150.
+// Against 128-bit arithmetic on random windows the error of r is at most 1.05 x 2^-53 of r (FP64
+// instructions: 2 to 4.4).
+__host__ __device__ __forceinline__ unsigned long long dmag_fixed(unsigned long long b, int right) {
+  return (((b & 0x000fffffffffffffULL) | 0x0010000000000000ULL) << 10) >> right;
+}
+__host__ __device__ __forceinline__ unsigned long long fixed_slope2(unsigned long long n, unsigned long long d) {
+  const unsigned long long m = 4 * (n < d ? n : d), s = n + d;
+  return s < m ? s : m;
+}
+// the double nearest to x 2^(e - 1082) with the sign bit `sign`, for x in [2^55, 2^60)
+__host__ __device__ __forceinline__ unsigned long long fixed_to_bits(unsigned long long x, int e,
+                                                                     unsigned long long sign) {
+  const unsigned hi = (unsigned)(x >> 32);
+#ifdef __CUDA_ARCH__
+  const int sh = 11 - __clz(hi);  // the leading bit is bit 32 + 31 - clz: to bit 52
+#else
+  const int sh = 11 - __builtin_clz(hi);
+#endif
+  return (((x + (1u << (sh - 1))) >> sh) + ((unsigned long long)(unsigned)(e - 8 + sh) << 52)) | sign;
+}
+// bit patterns of r and s from those of dl, d, dn, for the exponent field of d in [128, 2039] or
+// d = 0 (then both are 0)
+__host__ __device__ __forceinline__ void ppm_split_bits(unsigned long long bl, unsigned long long bd,
+                                                        unsigned long long bn, unsigned long long& r,
+                                                        unsigned long long& s) {
+  const int e = (int)(bd >> 52) & 0x7ff, el = (int)(bl >> 52) & 0x7ff, en = (int)(bn >> 52) & 0x7ff;
+  int kl = e - el + 3, kn = e - en + 3;
+  kl = kl < 0 ? 0 : (kl > 63 ? 63 : kl);
+  kn = kn < 0 ? 0 : (kn > 63 ? 63 : kn);
+  if ((long long)(bl ^ bd) < 0) kl = 63;
+  if ((long long)(bn ^ bd) < 0) kn = 63;
+  const unsigned long long fd = dmag_fixed(bd, 3);
+  const unsigned long long d0 = fixed_slope2(dmag_fixed(bl, kl), fd), d1 = fixed_slope2(dmag_fixed(bn, kn), fd);
+  // t / 12 with 2^64 / 12 = 0x15555555_55555555
+  const long long t = (long long)(d0 - d1);
+  const int th = (int)(t >> 32);
+  const unsigned tl = (unsigned)t;
+  const long long q = (long long)th * 0x15555555 + (long long)(((unsigned long long)tl * 0x15555555u) >> 32) +
+                      (((long long)th * 0x55555555) >> 32);
+  const unsigned long long x = (fd >> 1) + (unsigned long long)q;
+  const unsigned long long sign = bd & 0x8000000000000000ULL;
+  const bool zero = (bd << 1) == 0;
+  r = zero ? 0 : fixed_to_bits(x, e, sign);
+  s = zero ? 0 : fixed_to_bits(fd - x, e, sign);
+}
+__device__ __forceinline__ void ppm_split(double dl, double d, double dn, double& r, double& s) {
+  const unsigned long long bd = (unsigned long long)dbits(d);
+  const unsigned e = (unsigned)(bd >> 52) & 0x7ff;
+  if (e - 128u > 1911u && (bd << 1) != 0) {  // out of the fixed-point form's range
+    r = fma(vl_slope2(dl, d) - vl_slope2(d, dn), 1.0 / 12.0, halve(d));
+    s = d - r;
+    return;
+  }
+  unsigned long long br, bs;
+  ppm_split_bits((unsigned long long)dbits(dl), bd, (unsigned long long)dbits(dn), br, bs);
+  r = dfrom((long long)br);
+  s = dfrom((long long)bs);
+}
+
 template <> struct Rec<REC_PPM> {
-  static constexpr int LB = 3, LA = 2;
+  static constexpr int LB = 3, LA = 2, NS = 7, NB = 0;
   double q1, q2;      // q[m], q[m+1]
-  double dq;          // q[m+1] - q[m]
-  double d1;          // doubled slope of point m
+  double dl, dq;      // q[m] - q[m-1], q[m+1] - q[m]
+  double s2;          // q[m] - f1
   double f1;          // interface value at m - 1/2
   double aRprev;      // upper value of point m-1
+  int code;
+  template <class F> __device__ __forceinline__ void each(F f) {
+    f(0, q1);
+    f(1, q2);
+    f(2, dl);
+    f(3, dq);
+    f(4, s2);
+    f(5, f1);
+    f(6, aRprev);
+  }
   __device__ __forceinline__ void init(const double* v) {  // v = q[m0-3 .. m0+1]
     const double e0 = v[1] - v[0], e1 = v[2] - v[1], e2 = v[3] - v[2], e3 = v[4] - v[3];
-    const double da = vl_slope2(e0, e1);
-    const double db = vl_slope2(e1, e2);
-    const double dc = vl_slope2(e2, e3);
-    const double fa = ppm_iface(v[1], e1, da, db);
-    const double fb = ppm_iface(v[2], e2, db, dc);
-    double aL = fa, aR = fb;
-    ppm_mono(v[2], aL, aR);
+    double ra, sa, rb, sb;
+    ppm_split(e0, e1, e2, ra, sa);
+    ppm_split(e1, e2, e3, rb, sb);
+    const double fb = v[2] + rb;
+    double aL = v[1] + ra, aR = fb;
+    ppm_mono(v[2], rb, sa, aL, aR);
     aRprev = aR;
     q1 = v[3];
     q2 = v[4];
+    dl = e2;
     dq = e3;
-    d1 = dc;
+    s2 = sb;
     f1 = fb;
   }
   __device__ __forceinline__ void step(double qn, double& L, double& R) {
     const double dn = qn - q2;
-    const double d2 = vl_slope2(dq, dn);
-    const double f2 = ppm_iface(q1, dq, d1, d2);
+    double r, s;
+    ppm_split(dl, dq, dn, r, s);
+    const double f2 = q1 + r;
     double aL = f1, aR = f2;
-    ppm_mono(q1, aL, aR);
+    ppm_mono(q1, r, s2, aL, aR);
     L = aRprev;
     R = aL;
     aRprev = aR;
     q1 = q2;
     q2 = qn;
+    dl = dq;
     dq = dn;
-    d1 = d2;
+    s2 = s;
     f1 = f2;
   }
 };
@@ -394,70 +481,92 @@ __device__ __forceinline__ int median3_pick(T a, T b, T c) {
   const long long km = m == 2 ? kc : khi;
   return klo >= km ? lo : m;
 }
-template <class T>
-__device__ __forceinline__ T ppm_ep_iface(T qa, T qb, T qc, T qd) {
-  return fma(7.0 / 12.0, qa + qb, (qc + qd) * (-1.0 / 12.0));
-}
-// Interface between qa and qb (outer neighbours qc before qa, qd after qb); keep: it lies at a
-// smooth extremum (no bound). pick: 0 the fourth-order value, 1 qa, 2 qb.
-template <class T>
-__device__ __forceinline__ T ppm_ep_face(T qc, T qa, T qb, T qd, bool keep, int& pick) {
-  const T f = ppm_ep_iface(qa, qb, qc, qd);
+// The fourth-order value (7 (qa + qb) - (qc + qd)) / 12 lies r = d/2 + (dl - dn)/12 above qa, with
+// d = qb - qa and the differences dl before qa and dn after qb.
+// r and s = qb - f of the interface between qa and qb (f = qa + r); keep: it lies at a smooth
+// extremum (no bound), else f is bounded by the two cells. pick: 0 the fourth-order value, 1 qa, 2 qb.
+__device__ __forceinline__ double ppm_ep_face(double qa, double qb, double dl, double d, double dn, bool keep,
+                                              int& pick, double& r, double& s) {
+  r = fma(dl - dn, 1.0 / 12.0, halve(d));
+  s = d - r;
+  const double f = qa + r;
   pick = 0;
   if (!keep) {
     const int k = median3_pick(qa, f, qb);
     pick = k == 0 ? 1 : (k == 1 ? 0 : 2);
   }
+  if (pick != 0) {
+    r = pick == 1 ? 0.0 : d;
+    s = pick == 1 ? d : 0.0;
+  }
   return pick == 0 ? f : (pick == 1 ? qa : qb);
+}
+// sign code of a - b: a comparison (the rounded difference of two doubles has the sign of the exact
+// one)
+__device__ __forceinline__ int cmp_code(double a, double b) {
+  const long long ka = okey(a), kb = okey(b);
+  const bool z = is_zero(a) && is_zero(b);  // +0 and -0 are equal
+  return z ? 0 : ((int)(ka > kb) | ((int)(ka < kb) << 1));
 }
 
 template <> struct Rec<REC_PPM_EP> {
-  static constexpr int LB = 3, LA = 2;
-  double q0, q1, q2;  // q[m-1], q[m], q[m+1]
-  double dq;          // q[m+1] - q[m]
+  static constexpr int LB = 3, LA = 2, NS = 7, NB = 3;
+  double q1, q2;      // q[m], q[m+1]
+  double dl, dq;      // q[m] - q[m-1], q[m+1] - q[m]
+  double s2;          // q[m] - f1
   double f1;          // interface value at m - 1/2
   double aRprev;      // upper value of point m-1
-  // sign codes: bits 0-1 of q[m] - q[m-1], 2-3 and 4-5 of the curvatures of points m-1 and m;
-  // bit 6: interface m - 1/2 lies at an extremum
-  int code;
+  int code;           // bits 0-1: sign code of the curvature of point m-1; bit 2: interface m - 1/2
+                      // lies at an extremum
+  template <class F> __device__ __forceinline__ void each(F f) {
+    f(0, q1);
+    f(1, q2);
+    f(2, dl);
+    f(3, dq);
+    f(4, s2);
+    f(5, f1);
+    f(6, aRprev);
+  }
   __device__ __forceinline__ void init(const double* v) {  // v = q[m0-3 .. m0+1]
     const double e0 = v[1] - v[0], e1 = v[2] - v[1], e2 = v[3] - v[2], e3 = v[4] - v[3];
-    const int s0 = sgn_code(e0), s1 = sgn_code(e1), s2 = sgn_code(e2), s3 = sgn_code(e3);
+    const int s0 = sgn_code(e0), s1 = sgn_code(e1), sb = sgn_code(e2), s3 = sgn_code(e3);
     // curvature codes of points m0-2, m0-1, m0
-    const int ka = sgn_code(e1 - e0), kb = sgn_code(e2 - e1), kc = sgn_code(e3 - e2);
-    const bool xa = ext_code(s0, s1, s2), xb = ext_code(s1, s2, s3);
+    const int ka = cmp_code(e1, e0), kb = cmp_code(e2, e1), kc = cmp_code(e3, e2);
+    const bool xa = ext_code(s0, s1, sb), xb = ext_code(s1, sb, s3);
     int p;
-    const double fa = ppm_ep_face(v[0], v[1], v[2], v[3], xa && same_code(ka, kb), p);  // m0 - 3/2
-    const double fb = ppm_ep_face(v[1], v[2], v[3], v[4], xb && same_code(kb, kc), p);  // m0 - 1/2
+    double ra, sa, rb;
+    const double fa = ppm_ep_face(v[1], v[2], e0, e1, e2, xa && same_code(ka, kb), p, ra, sa);   // m0 - 3/2
+    const double fb = ppm_ep_face(v[2], v[3], e1, e2, e3, xb && same_code(kb, kc), p, rb, s2);  // m0 - 1/2
     double aL = fa, aR = fb;
-    if (!((xa || xb) && same_code(ka, kb) && same_code(kb, kc))) ppm_mono(v[2], aL, aR);
+    if (!((xa || xb) && same_code(ka, kb) && same_code(kb, kc))) ppm_mono(v[2], rb, sa, aL, aR);
     aRprev = aR;
-    q0 = v[2];
     q1 = v[3];
     q2 = v[4];
+    dl = e2;
     dq = e3;
     f1 = fb;
-    code = s2 | (kb << 2) | (kc << 4) | ((int)xb << 6);
+    code = kb | ((int)xb << 2);
   }
   __device__ __forceinline__ void step(double qn, double& L, double& R) {
     const double dn = qn - q2;  // q[m+2] - q[m+1]
-    const int sm = code & 3, c0 = (code >> 2) & 3, c1 = (code >> 4) & 3;
-    const bool x1 = code >> 6;
-    const int s0 = sgn_code(dq), sp = sgn_code(dn), cn = sgn_code(dn - dq);  // cn: point m+1
-    const bool x2 = ext_code(sm, s0, sp);
+    const int c0 = code & 3, c1 = cmp_code(dq, dl), cn = cmp_code(dn, dq);  // points m-1, m, m+1
+    const bool x1 = code >> 2;
+    const bool x2 = ext_code(sgn_code(dl), sgn_code(dq), sgn_code(dn));
     int p;
-    const double f2 = ppm_ep_face(q0, q1, q2, qn, x2 && same_code(c1, cn), p);  // m + 1/2
+    double r, s;
+    const double f2 = ppm_ep_face(q1, q2, dl, dq, dn, x2 && same_code(c1, cn), p, r, s);  // m + 1/2
     double aL = f1, aR = f2;
-    if (!((x1 || x2) && same_code(c0, c1) && same_code(c1, cn))) ppm_mono(q1, aL, aR);
+    if (!((x1 || x2) && same_code(c0, c1) && same_code(c1, cn))) ppm_mono(q1, r, s2, aL, aR);
     L = aRprev;
     R = aL;
     aRprev = aR;
-    q0 = q1;
     q1 = q2;
     q2 = qn;
+    dl = dq;
     dq = dn;
+    s2 = s;
     f1 = f2;
-    code = s0 | (c1 << 2) | (cn << 4) | ((int)x2 << 6);
+    code = c1 | ((int)x2 << 2);
   }
 };
 

@@ -5,14 +5,9 @@
 
 namespace mhd {
 
-// blocks of 128 threads the compiler must fit per SM (register budget of the face sweep)
-#ifndef MHD_FACE_MINB
-#define MHD_FACE_MINB 1
-#endif
-
 // one direction, one thread per segment (the form without work cursors: mhd_step_noalloc)
 template <int RC, int RS>
-__global__ void __launch_bounds__(128, MHD_FACE_MINB) k_face(Dev D, int dir, int seg) {
+__global__ void __launch_bounds__(kFaceThreads, kFaceMinBlocks) k_face(Dev D, int dir, int seg) {
   Line ln;
   int m0, m1;
   if (!sweep_line(D, dir, seg, ln, m0, m1)) return;
@@ -25,7 +20,7 @@ __global__ void __launch_bounds__(128, MHD_FACE_MINB) k_face(Dev D, int dir, int
 // run while the other SMs idle). A warp's 32 segments lie on an 8 x 4 patch of lines where the box
 // allows (sweep_line_at), so that its lanes take the same Riemann-fan branch more often.
 template <int RC, int RS>
-__global__ void __launch_bounds__(128, MHD_FACE_MINB) k_faces(Dev D, int s0, int s1, int s2) {
+__global__ void __launch_bounds__(kFaceThreads, kFaceMinBlocks) k_faces(Dev D, int s0, int s1, int s2) {
   const long long t0 = sweep_threads(D, 0, s0), t1 = sweep_threads(D, 1, s1), t2 = sweep_threads(D, 2, s2);
   for_each_segment(D.work, t0 + t1 + t2, [&](long long t) {
     int dir = 0, seg = s0;
@@ -47,8 +42,8 @@ __global__ void __launch_bounds__(128, MHD_FACE_MINB) k_faces(Dev D, int s0, int
 
 template <int RC, int RS>
 static void launch_faces_t(const Dev& d, int seg, cudaStream_t st) {
-  const int bs = 128;
-  const long long res = resident_blocks((const void*)k_faces<RC, RS>, bs);
+  const int bs = kFaceThreads, smem = face_smem_bytes<RC>();
+  const long long res = resident_blocks((const void*)k_faces<RC, RS>, bs, smem);
   int sg[3];
   long long tot = 0;
   for (int dir = 0; dir < 3; ++dir) {
@@ -57,14 +52,15 @@ static void launch_faces_t(const Dev& d, int seg, cudaStream_t st) {
   }
   const long long blocks = std::min((tot + bs - 1) / bs, res);
   cudaMemsetAsync(d.work, 0, sizeof(unsigned long long), st);
-  k_faces<RC, RS><<<(unsigned)blocks, bs, 0, st>>>(d, sg[0], sg[1], sg[2]);
+  k_faces<RC, RS><<<(unsigned)blocks, bs, smem, st>>>(d, sg[0], sg[1], sg[2]);
 }
 
 template <int RC, int RS>
 static void launch_face_t(const Dev& d, int dir, int seg, cudaStream_t st) {
-  const int bs = 128;
+  const int bs = kFaceThreads, smem = face_smem_bytes<RC>();
   const long long threads = sweep_threads(d, dir, seg);
-  k_face<RC, RS><<<(unsigned)((threads + bs - 1) / bs), bs, 0, st>>>(d, dir, seg);
+  resident_blocks((const void*)k_face<RC, RS>, bs, smem);  // (allows the kernel its shared memory)
+  k_face<RC, RS><<<(unsigned)((threads + bs - 1) / bs), bs, smem, st>>>(d, dir, seg);
 }
 
 template <int RC>

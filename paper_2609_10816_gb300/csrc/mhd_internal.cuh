@@ -103,8 +103,9 @@ void launch_vjp_check(long long n, unsigned long long seed, double gam, int rs, 
                       cudaStream_t st);
 
 // blocks of `threads` threads of kernel `fn` that fit on the device at once (all SMs), for the
-// persistent launches of the dynamically scheduled sweeps; cached per kernel
-int resident_blocks(const void* fn, int threads);
+// persistent launches of the dynamically scheduled sweeps, with `smem` bytes of dynamic shared
+// memory each (which the kernel is then allowed to use); cached per kernel
+int resident_blocks(const void* fn, int threads, int smem = 0);
 
 // message reported by mhd_create_error() for calls that have no context
 void set_call_error(const char* msg);
