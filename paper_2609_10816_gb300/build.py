@@ -11,6 +11,10 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmhd.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
+# The forward kernels write every fused multiply-add they want as fma(): left to the compiler, which
+# product of a sum is fused depends on the kernel around it, and the single-box, batched and
+# allocation-free kernels give the same bits from the same device functions.
+NO_CONTRACTION = ("mhd_face", "mhd_edge", "mhd_cell", "mhd_batch")
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
 
@@ -41,7 +45,8 @@ def build(force: bool = False, verbose: bool = False, extra: list | None = None)
         obj = os.path.join(OBJ, os.path.basename(src)[:-3] + ".o")
         if not force and os.path.exists(obj) and os.path.getmtime(obj) > max(os.path.getmtime(src), hm):
             return obj
-        cmd = [nvcc, *ARCH, *FLAGS, *extra, "-c", src, "-o", obj]
+        own = ["-fmad=false"] if os.path.basename(src).startswith(NO_CONTRACTION) else []
+        cmd = [nvcc, *ARCH, *FLAGS, *own, *extra, "-c", src, "-o", obj]
         if verbose:
             print(" ".join(cmd), file=sys.stderr)
         subprocess.check_call(cmd)

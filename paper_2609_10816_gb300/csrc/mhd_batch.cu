@@ -222,7 +222,13 @@ mhd_status upload_schedule(mhd_batch* b) {
     for (int d = 0; d < 3; ++d) {
       const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
       const long long segs = (n[d] + b->seg - 1) / b->seg;
-      sp[d * (np + 1) + k + 1] = sp[d * (np + 1) + k] + (long long)n[t1] * n[t2] * segs;
+      long long c = (long long)n[t1] * n[t2] * segs;
+      if (d == 0) {  // the face phase's sweep along x: whole warps (items of lane sweeps)
+        mhd::Dev D;
+        for (int j = 0; j < 3; ++j) D.n[j] = n[j];
+        c = mhd::face_by_lanes(D, 0) ? mhd::lane_threads(D, 0, mhd::lane_seg(b->seg)) : (c + 31) / 32 * 32;
+      }
+      sp[d * (np + 1) + k + 1] = sp[d * (np + 1) + k] + c;
     }
     // the edge phases' segments along x: edge_sweep_seg's length, about nx / 32 points (4 to 16)
     const int sx = std::min(16, std::max(4, (n[0] + 31) / 32));

@@ -16,7 +16,8 @@ struct BatchDev {
   const int* order;               // patch visited at schedule position k, [npatch]
   const long long* cell_pref;     // [npatch + 1] cells before schedule position k
   const long long* sweep_pref;    // [4][npatch + 1] sweep segments along dir (row 3: the edge sweeps'
-                                  // segments along x) before position k
+                                  // segments along x) before position k; row 0 in multiples of 32
+                                  // (a lane sweep's item is 32 of them)
   int npatch;
   int seg;
   int stage;
@@ -93,11 +94,9 @@ __device__ inline bool grid_sync(const BatchDev& B) {
 
 // One sweep phase: the sweeps along dirs[0..2] of every patch form one work list (sweep j's
 // segments after those of sweeps 0 .. j-1, patches in schedule order), taken 32 segments at a
-// time per warp from `cursor`; fn(D, j, line, m0, m1) runs each segment. In the edge phases
-// (EDGE) the lines along x are cut as the single-box edge sweeps cut them: short segments
-// numbered along the line, so that a warp walks whole lines (one thread per x-line would stream
-// a separate cache line per thread and array).
-template <bool EDGE = false, class Fn>
+// time per warp from `cursor`; fn(D, j, t) runs segment t of a patch's sweep j. In the edge phases
+// (EDGE) the sweeps along x have segments of their own.
+template <bool EDGE, class Fn>
 __device__ __forceinline__ void sweep_phase(const BatchDev& B, unsigned long long* cursor, const int* dirs, Fn fn) {
   const long long* pref[3];
   long long tot[3];
@@ -117,12 +116,20 @@ __device__ __forceinline__ void sweep_phase(const BatchDev& B, unsigned long lon
       }
     }
     const int k = find_pos(pref[j], B.npatch, t);
-    const Dev& D = B.patches[B.order[k]];
-    const bool xl = EDGE && dirs[j] == 0;
+    fn(B.patches[B.order[k]], j, t - pref[j][k]);
+  });
+}
+// An edge phase: fn(D, j, line, m0, m1) runs each segment. The lines along x are cut as the
+// single-box edge sweeps cut them: short segments numbered along the line, so that a warp walks
+// whole lines (one thread per x-line would stream a separate cache line per thread and array);
+// along y and z warps lie on 8 x 4 patches of lines, as in the single-box sweeps.
+template <class Fn>
+__device__ __forceinline__ void edge_phase(const BatchDev& B, unsigned long long* cursor, const int* dirs, Fn fn) {
+  sweep_phase<true>(B, cursor, dirs, [&](const Dev& D, int j, long long t) {
+    const bool xl = dirs[j] == 0;
     Line ln;
     int m0, m1;
-    // (warps on 8 x 4 patches of lines, as in the single-box sweeps)
-    if (sweep_line_at(D, dirs[j], xl ? edge_sweep_seg(D, 0, B.seg) : B.seg, t - pref[j][k], ln, m0, m1, xl, !xl))
+    if (sweep_line_at(D, dirs[j], xl ? edge_sweep_seg(D, 0, B.seg) : B.seg, t, ln, m0, m1, xl, !xl))
       fn(D, j, ln, m0, m1);
   });
 }
@@ -188,8 +195,9 @@ __device__ __forceinline__ bool face_part(const BatchDev& B) {
   stamp(B, 1);
   // face sweeps along each direction
   const int dirs[3] = {0, 1, 2};
-  sweep_phase(B, B.cursor + 0, dirs, [&](const Dev& D, int j, const Line& ln, int m0, int m1) {
-    face_seg<RC, RS>(D, j, ln, m0, m1);
+  sweep_phase<false>(B, B.cursor + 0, dirs, [&](const Dev& D, int j, long long t) {
+    const bool lanes = face_by_lanes(D, j);
+    face_thread<RC, RS>(D, j, lanes, lanes ? lane_seg(B.seg) : B.seg, t);
   });
   return true;
 }
@@ -209,10 +217,10 @@ __device__ __forceinline__ bool rest_part(const BatchDev& B) {
     // the cell-centred EMF reconstructed to the a-faces (lines along a = e + 1) and to the c-faces
     // (lines along c = e + 2): two independent work lists, no barrier between them
     const int dirs_a[3] = {1, 2, 0}, dirs_c[3] = {2, 0, 1};
-    sweep_phase<true>(B, B.cursor + 3, dirs_a, [&](const Dev& D, int e, const Line& ln, int m0, int m1) {
+    edge_phase(B, B.cursor + 3, dirs_a, [&](const Dev& D, int e, const Line& ln, int m0, int m1) {
       b25_seg<RC>(D, e, 1, ln, m0, m1);
     });
-    sweep_phase<true>(B, B.cursor + 4, dirs_c, [&](const Dev& D, int e, const Line& ln, int m0, int m1) {
+    edge_phase(B, B.cursor + 4, dirs_c, [&](const Dev& D, int e, const Line& ln, int m0, int m1) {
       b25_seg<RC>(D, e, 0, ln, m0, m1);
     });
     if (!grid_sync(B)) return false;
@@ -220,7 +228,7 @@ __device__ __forceinline__ bool rest_part(const BatchDev& B) {
   // a-face quantities to e-edges (lines along c = e + 2)
   {
     const int dirs[3] = {2, 0, 1};
-    sweep_phase<true>(B, B.cursor + 1, dirs, [&](const Dev& D, int e, const Line& ln, int m0, int m1) {
+    edge_phase(B, B.cursor + 1, dirs, [&](const Dev& D, int e, const Line& ln, int m0, int m1) {
       edge_bt_seg<RC, EMF>(D, e, ln, m0, m1);
     });
   }
@@ -229,7 +237,7 @@ __device__ __forceinline__ bool rest_part(const BatchDev& B) {
   // c-face quantities to e-edges (lines along a = e + 1) and the edge EMFs
   {
     const int dirs[3] = {1, 2, 0};
-    sweep_phase<true>(B, B.cursor + 2, dirs, [&](const Dev& D, int e, const Line& ln, int m0, int m1) {
+    edge_phase(B, B.cursor + 2, dirs, [&](const Dev& D, int e, const Line& ln, int m0, int m1) {
       edge_lr_seg<RC, EMF>(D, e, ln, m0, m1);
     });
   }
@@ -333,22 +341,19 @@ __device__ __forceinline__ void fofc_part(const BatchDev& B) {
 // The stage's launches. One launch per stage runs every phase at the face sweep's register
 // budget; three launches per stage run the edge, update and flag phases at half that budget (twice
 // the warps per SM) and the first-order correction apart.
-template <int RC, int RS, int EMF>
-__device__ __forceinline__ void stage_all(const BatchDev& B) {
-  if (!face_part<RC, RS>(B)) return;
-  if (!grid_sync(B)) return;
-  if (!rest_part<RC, EMF, kCellIlp>(B)) return;
-  if (!B.fofc) return;
-  if (!grid_sync(B)) return;
-  fofc_part(B);
-}
 template <int RC, int RS>
 __global__ void __launch_bounds__(kFaceThreads, kStageMinBlocks) k_batch_stage(BatchDev B) {
+  if (!face_part<RC, RS>(B)) return;
+  if (!grid_sync(B)) return;
+  bool ok;
   switch (B.emf) {  // uniform over the grid
-    case EMF_FS18: stage_all<RC, RS, EMF_FS18>(B); break;
-    case EMF_B25A: stage_all<RC, RS, EMF_B25A>(B); break;
-    default: stage_all<RC, RS, EMF_Q26>(B); break;
+    case EMF_FS18: ok = rest_part<RC, EMF_FS18, kCellIlp>(B); break;
+    case EMF_B25A: ok = rest_part<RC, EMF_B25A, kCellIlp>(B); break;
+    default: ok = rest_part<RC, EMF_Q26, kCellIlp>(B); break;
   }
+  if (!ok || !B.fofc) return;
+  if (!grid_sync(B)) return;
+  fofc_part(B);
 }
 template <int RC, int RS>
 __global__ void __launch_bounds__(kFaceThreads, kFaceMinBlocks) k_batch_face(BatchDev B) {

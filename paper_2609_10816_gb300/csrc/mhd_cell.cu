@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(256) k_divb(Dev D, Ptr3 Bp, unsigned long long
     double acc = 0.0;
     for (int d = 0; d < 3; ++d) {
       const double lo = Bp.p[d][X], hi = Bp.p[d][shift(D, X, d, 1)];
-      acc += (hi - lo) * D.hinv[d];
+      acc = fma(hi - lo, D.hinv[d], acc);
       mb = pmax(mb, vabs(lo));
     }
     dv = vabs(acc);

@@ -258,8 +258,8 @@ __device__ __forceinline__ void fo_faces_cell(const Dev& D, long long X) {
       // Joule flux from the S^n field (same reading as the high-order faces)
       auto jedge = [&](int e, long long Y) {
         const int ae = (e + 1) % 3, ce = (e + 2) % 3;
-        return (D.B0[ce][Y] - D.B0[ce][shift(D, Y, ae, -1)]) * D.hinv[ae] -
-               (D.B0[ae][Y] - D.B0[ae][shift(D, Y, ce, -1)]) * D.hinv[ce];
+        return fma(D.B0[ce][Y] - D.B0[ce][shift(D, Y, ae, -1)], D.hinv[ae],
+                   -((D.B0[ae][Y] - D.B0[ae][shift(D, Y, ce, -1)]) * D.hinv[ce]));
       };
       const long long Xc = shift(D, X, c, 1), Xa = shift(D, X, a, 1);
       const double ea = 0.5 * D.eta * (jedge(a, X) + jedge(a, Xc));
@@ -323,7 +323,7 @@ __device__ __forceinline__ void fo_edges_cell(const Dev& D, long long X) {
     const double up = fma(apc, fma(apa, eLB, apa * eRB), apc * fma(apa, eLT, apa * eRT)) * (ia * ic);
     double emf = fma(apa * apa * ia, bcR - bcL, fma(-apc * apc * ic, baT - baB, up));
     if (D.resistive) {
-      const double j = (D.B0[c][X] - D.B0[c][Xa]) * D.hinv[a] - (D.B0[a][X] - D.B0[a][Xc]) * D.hinv[c];
+      const double j = fma(D.B0[c][X] - D.B0[c][Xa], D.hinv[a], -((D.B0[a][X] - D.B0[a][Xc]) * D.hinv[c]));
       emf = fma(D.eta, j, emf);
     }
     D.E[e * N + X] = emf;

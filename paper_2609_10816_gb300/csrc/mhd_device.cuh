@@ -571,6 +571,99 @@ template <> struct Rec<REC_PPM_EP> {
 };
 
 // ------------------------------------------------------------------------------------------
+// The same reconstructions with a warp's lanes along the line: a lane holds face m (between points
+// m - 1 and m), the lane before it face m - 1, and what a walk would carry from face to face comes
+// from the lanes before, across a pass of 8 faces from the previous pass's values. step() takes the
+// points m .. m + LA (PC: m - 1 and m), prev[NP] with this lane's values of the previous pass
+// (replaced by those of this pass) and returns the interface's states. The values are those of Rec
+// bit for bit. Every lane of the warp calls it. One pass of 8 points ahead of the first face fills
+// prev (its own prev may hold anything).
+// ------------------------------------------------------------------------------------------
+struct LaneWalk {
+  int k;           // this lane's place in its row of 8
+  int src1, src2;  // the lanes that hold places k - 1 and k - 2 (mod 8)
+  __device__ __forceinline__ double up1(double cur, double prev) const {
+    return __shfl_sync(0xffffffffu, k == 7 ? prev : cur, src1);
+  }
+  __device__ __forceinline__ double up2(double cur, double prev) const {
+    return __shfl_sync(0xffffffffu, k >= 6 ? prev : cur, src2);
+  }
+  __device__ __forceinline__ int up1(int cur, int prev) const {
+    return __shfl_sync(0xffffffffu, k == 7 ? prev : cur, src1);
+  }
+};
+template <int R> struct LaneRec;
+template <> struct LaneRec<REC_PC> {
+  static constexpr int NP = 0, FIRST = -1, NQ = 2, NB = 0;
+  __device__ __forceinline__ static void step(const LaneWalk&, const double* q, double*, int&, double& L, double& R) {
+    L = q[0];
+    R = q[1];
+  }
+};
+template <int RC> struct LanePLM {
+  static constexpr int NP = 2, FIRST = 0, NQ = 2, NB = 0;
+  __device__ __forceinline__ static void step(const LaneWalk& w, const double* q, double* prev, int&, double& L,
+                                              double& R) {
+    const double dr = q[1] - q[0];
+    const double dl = w.up1(dr, prev[0]);
+    const double h = RC == REC_PLM_MC ? half_slope_mc(dl, dr) : half_slope_minmod(dl, dr);
+    const double aR = q[0] + h;
+    L = w.up1(aR, prev[1]);
+    R = q[0] - h;
+    prev[0] = dr;
+    prev[1] = aR;
+  }
+};
+template <> struct LaneRec<REC_PLM_MC> : LanePLM<REC_PLM_MC> {};
+template <> struct LaneRec<REC_PLM_MINMOD> : LanePLM<REC_PLM_MINMOD> {};
+template <> struct LaneRec<REC_PPM> {
+  static constexpr int NP = 4, FIRST = 0, NQ = 3, NB = 0;
+  __device__ __forceinline__ static void step(const LaneWalk& w, const double* q, double* prev, int&, double& L,
+                                              double& R) {
+    const double dn = q[2] - q[1];
+    const double dq = w.up1(dn, prev[0]), dl = w.up2(dn, prev[0]);
+    double r, s;
+    ppm_split(dl, dq, dn, r, s);
+    const double f2 = q[0] + r;
+    const double s2 = w.up1(s, prev[1]);
+    double aL = w.up1(f2, prev[2]), aR = f2;
+    ppm_mono(q[0], r, s2, aL, aR);
+    L = w.up1(aR, prev[3]);
+    R = aL;
+    prev[0] = dn;
+    prev[1] = s;
+    prev[2] = f2;
+    prev[3] = aR;
+  }
+};
+template <> struct LaneRec<REC_PPM_EP> {
+  static constexpr int NP = 4, FIRST = 0, NQ = 3, NB = 3;
+  __device__ __forceinline__ static void step(const LaneWalk& w, const double* q, double* prev, int& code, double& L,
+                                              double& R) {
+    const double dn = q[2] - q[1];
+    const double dq = w.up1(dn, prev[0]), dl = w.up2(dn, prev[0]);
+    const int c1 = cmp_code(dq, dl), cn = cmp_code(dn, dq);  // curvatures of points m, m + 1
+    const bool x2 = ext_code(sgn_code(dl), sgn_code(dq), sgn_code(dn));
+    int p;
+    double r, s;
+    const double f2 = ppm_ep_face(q[0], q[1], dl, dq, dn, x2 && same_code(c1, cn), p, r, s);
+    const double s2 = w.up1(s, prev[1]);
+    double aL = w.up1(f2, prev[2]), aR = f2;
+    const int mine = c1 | ((int)x2 << 2), before = w.up1(mine, code);
+    const int c0 = before & 3;
+    const bool x1 = before >> 2;
+    if (!((x1 || x2) && same_code(c0, c1) && same_code(c1, cn))) ppm_mono(q[0], r, s2, aL, aR);
+    L = w.up1(aR, prev[3]);
+    R = aL;
+    prev[0] = dn;
+    prev[1] = s;
+    prev[2] = f2;
+    prev[3] = aR;
+    code = mine;
+  }
+};
+
+// ------------------------------------------------------------------------------------------
 // Riemann problem on one face, in the face frame (n, t1, t2).
 // W = {rho, u_n, u_t1, u_t2, p, b_t1, b_t2}; bn = stored face field.
 // ------------------------------------------------------------------------------------------

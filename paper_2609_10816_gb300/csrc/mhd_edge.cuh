@@ -273,7 +273,7 @@ __device__ __forceinline__ void edge_lr_seg(const Dev& D, int e, const Line& ln,
     }
     if (EMF != EMF_Q26) emf = ld04(apa, ama, apc, amc, eLB, eRB, eLT, eRT, baB, baT, bcL, bcR);
     if (D.resistive) {
-      const double j = (Bc[X] - Bc[Xa]) * D.hinv[a] - (Ba[X] - Ba[Xc]) * D.hinv[c];
+      const double j = fma(Bc[X] - Bc[Xa], D.hinv[a], -((Ba[X] - Ba[Xc]) * D.hinv[c]));
       emf = fma(D.eta, j, emf);
     }
     E[X] = D.combine ? halve(E[X] + emf) : emf;

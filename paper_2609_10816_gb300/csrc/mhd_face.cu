@@ -11,17 +11,21 @@ __global__ void __launch_bounds__(kFaceThreads, kFaceMinBlocks) k_face(Dev D, in
   Line ln;
   int m0, m1;
   if (!sweep_line(D, dir, seg, ln, m0, m1)) return;
-  face_seg<RC, RS>(D, dir, ln, m0, m1);
+  face_piece<RC, RS>(D, dir, false, ln, m0, m1, LaneWalk{0, 0, 0}, true);
 }
 
 // The three face sweeps of a stage as one persistent launch: the segments of the x, y and z
 // sweeps form one work list behind one cursor, so that the grid drains one tail per stage instead
 // of one per direction (a warp takes 32 segments of up to 64 faces at a time, and the last ones
 // run while the other SMs idle). A warp's 32 segments lie on an 8 x 4 patch of lines where the box
-// allows (sweep_line_at), so that its lanes take the same Riemann-fan branch more often.
+// allows (sweep_line_at), so that its lanes take the same Riemann-fan branch more often. Each
+// direction's part of the list starts at a multiple of 32, so that an item of a lane sweep is one
+// warp's.
+__device__ __forceinline__ long long round32(long long t) { return (t + 31) / 32 * 32; }
 template <int RC, int RS>
-__global__ void __launch_bounds__(kFaceThreads, kFaceMinBlocks) k_faces(Dev D, int s0, int s1, int s2) {
-  const long long t0 = sweep_threads(D, 0, s0), t1 = sweep_threads(D, 1, s1), t2 = sweep_threads(D, 2, s2);
+__global__ void __launch_bounds__(kFaceThreads, kFaceMinBlocks) k_faces(Dev D, int s0, int s1, int s2, int x_lanes) {
+  const long long t0 = x_lanes ? lane_threads(D, 0, s0) : round32(sweep_threads(D, 0, s0));
+  const long long t1 = round32(sweep_threads(D, 1, s1)), t2 = round32(sweep_threads(D, 2, s2));
   for_each_segment(D.work, t0 + t1 + t2, [&](long long t) {
     int dir = 0, seg = s0;
     if (t >= t0) {
@@ -34,25 +38,35 @@ __global__ void __launch_bounds__(kFaceThreads, kFaceMinBlocks) k_faces(Dev D, i
         seg = s2;
       }
     }
-    Line ln;
-    int m0, m1;
-    if (sweep_line_at(D, dir, seg, t, ln, m0, m1, false, true)) face_seg<RC, RS>(D, dir, ln, m0, m1);
+    face_thread<RC, RS>(D, dir, x_lanes && dir == 0, seg, t);
   });
 }
 
+// Boxes below this many cells walk the x sweep too: they have too few segments to pay for the pass
+// that fills a lane sweep's windows (32^3, PLM + HLL: face sweeps of a step 114 us walked, 151 by
+// lanes; 64^3, PPM + HLLD, one stage with stored states: 388 against 384).
+constexpr long long kLaneCells = 1LL << 17;
 template <int RC, int RS>
 static void launch_faces_t(const Dev& d, int seg, cudaStream_t st) {
   const int bs = kFaceThreads, smem = face_smem_bytes<RC>();
   const long long res = resident_blocks((const void*)k_faces<RC, RS>, bs, smem);
   int sg[3];
   long long tot = 0;
+  const bool x_lanes = face_by_lanes(d, 0) && d.N >= kLaneCells;
   for (int dir = 0; dir < 3; ++dir) {
-    sg[dir] = fill_seg(d, dir, seg, res * bs);
-    tot += sweep_threads(d, dir, sg[dir]);
+    if (dir == 0 && x_lanes) {
+      // whole passes of 8; two items per resident warp, as fill_seg does for the others
+      sg[dir] = lane_seg(2 * seg);
+      while (sg[dir] > 8 && lane_threads(d, dir, sg[dir]) < 2 * res * bs) sg[dir] = lane_seg(sg[dir] / 2);
+      tot += lane_threads(d, dir, sg[dir]);
+    } else {
+      sg[dir] = fill_seg(d, dir, seg, res * bs);
+      tot += sweep_threads(d, dir, sg[dir]) + 31;
+    }
   }
   const long long blocks = std::min((tot + bs - 1) / bs, res);
   cudaMemsetAsync(d.work, 0, sizeof(unsigned long long), st);
-  k_faces<RC, RS><<<(unsigned)blocks, bs, smem, st>>>(d, sg[0], sg[1], sg[2]);
+  k_faces<RC, RS><<<(unsigned)blocks, bs, smem, st>>>(d, sg[0], sg[1], sg[2], x_lanes ? 1 : 0);
 }
 
 template <int RC, int RS>

@@ -103,6 +103,20 @@ __device__ __forceinline__ bool sweep_line(const Dev& D, int dir, int seg, Line&
   return sweep_line_at(D, dir, seg, (long long)blockIdx.x * blockDim.x + threadIdx.x, ln, m0, m1, seg_fastest);
 }
 
+// Lane sweeps: a warp takes 8 consecutive points of 4 neighbouring lines at a time and walks them
+// 8 points further per pass, handing the sliding windows' state from lane to lane by shuffles. An
+// item is one such group of lines over one segment of `seg` points (a multiple of 8); 32 threads
+// of a work list stand for it.
+__host__ __device__ __forceinline__ int lane_seg(int seg) { return seg < 8 ? 8 : (seg + 7) / 8 * 8; }
+__host__ __device__ __forceinline__ long long lane_groups(const Dev& D, int dir) {
+  int t1, t2;
+  sweep_axes(dir, t1, t2);
+  return ((long long)D.n[t1] * D.n[t2] + 3) / 4;
+}
+__host__ __device__ __forceinline__ long long lane_threads(const Dev& D, int dir, int seg) {
+  return 32 * lane_groups(D, dir) * ((D.n[dir] + seg - 1) / seg);
+}
+
 // Dynamic schedule of a sweep: a persistent grid whose warps each take the next 32 segments of the
 // work list from a cursor in device memory until the list is exhausted, so that no SM idles while
 // others finish a long tail (segments differ in cost through the Riemann-fan and limiter branches).
