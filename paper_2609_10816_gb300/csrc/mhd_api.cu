@@ -292,8 +292,7 @@ static mhd_status advance(mhd_ctx* ctx, const mhd_state* state, mhd::Dev D, cons
                           bool prim_ready = false) {
   const long long N = D.N;
   mhd_status s;
-  D.eta = eta;
-  D.resistive = eta != 0.0;
+  mhd::set_eta(D, eta);
   D.emf = sc.emf;
   if (!sc.fofc) D.fofc_criteria = 0;  // flags then count only non-finite cells
   D.U0 = state->cons;
@@ -357,6 +356,7 @@ namespace {
 // the launches of one mhd_step_cfl on ctx->stream: CFL reduction, dt, both stages
 mhd_status enqueue_step_cfl(mhd_ctx* ctx, const mhd_state* state, double cfl, const Decoded& sc, double eta) {
   mhd::Dev D = ctx->base;
+  mhd::set_eta(D, eta);  // (the reduction also leaves the currents of S^n)
   cudaStream_t st = ctx->stream;
   mhd_status s = cuda_check(ctx, cudaMemsetAsync(D.counters + 2, 0, sizeof(unsigned long long), st),
                             "cudaMemsetAsync");
@@ -595,7 +595,7 @@ mhd_status mhd_step_adjoint(mhd_ctx* ctx, const mhd_state* state, const mhd_stat
   mhd::Dev D = ctx->base;
   D.dt = dt;
   for (int d = 0; d < 3; ++d) D.dth[d] = dt * D.hinv[d];
-  D.eta = eta;
+  mhd::set_eta(D, eta);
   // the resistive terms are linear in eta: their derivative in eta is needed even at eta = 0,
   // where they add exact zeros to the forward values
   D.resistive = 1;

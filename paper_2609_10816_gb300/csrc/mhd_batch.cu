@@ -262,8 +262,7 @@ mhd_status upload_params(mhd_batch* b, const mhd_batch_state* s, int scheme, dou
     for (int d = 0; d < 3; ++d) { D.h[d] = b->h; D.hinv[d] = 1.0 / b->h; }
     D.gam = b->gamma;
     D.gm1inv = 1.0 / (b->gamma - 1.0);
-    D.eta = eta;
-    D.resistive = eta != 0.0;
+    mhd::set_eta(D, eta);
     D.fofc_criteria = (scheme & MHD_FOFC_OFF) ? 0 : 3;
     D.emf = (scheme >> 8) & 0xf;
     if (D.emf != mhd::EMF_Q26) {

@@ -188,8 +188,10 @@ __device__ __forceinline__ bool face_part(const BatchDev& B) {
     }
 #pragma unroll
     for (int g = 0; g < kCellIlp; ++g)
-      if (Dp[g])
+      if (Dp[g]) {
         for (int v = 0; v < 8; ++v) Dp[g]->P[v * Dp[g]->N + X[g]] = w[g][v];
+        store_current(*Dp[g], Dp[g]->Bin, X[g]);
+      }
   }
   if (!grid_sync(B)) return false;
   stamp(B, 1);
@@ -299,8 +301,10 @@ __device__ __forceinline__ bool rest_part(const BatchDev& B) {
                             : invalid_vals(*Dp[g], u[g], lo[g], hi[g]);
         Dp[g]->flag[X[g]] = f[g] ? 1 : 0;
         if (f[g]) atomicAdd(&pflags[K[g]], 1u);
-        if (B.stage == 0)  // the primitives of S^{n+1/2}, stage 2's input
+        if (B.stage == 0) {  // the primitives and currents of S^{n+1/2}, stage 2's input
           for (int v = 0; v < 8; ++v) Dp[g]->P[v * Dp[g]->N + X[g]] = pw[g][v];
+          store_current(*Dp[g], Dp[g]->Bout, X[g]);
+        }
       }
       cnt += __popc(__ballot_sync(0xffffffffu, f[g]));
     }

@@ -25,25 +25,18 @@
 namespace mhd {
 
 // Joule flux eta (j x b)_d on the d-face of cell X (reading: eta j from the mean of the face's
-// two bounding edges per tangential direction, tangential b from the four nearest faces).
+// two bounding edges per tangential direction, tangential b from the four nearest faces, which is
+// the mean of the two cells' b). The edges' eta j / 2 were left with the primitives (store_current).
 __device__ __forceinline__ double joule_flux(const Dev& D, int d, long long X) {
   const int a = (d + 1) % 3, c = (d + 2) % 3;
-  const double* Ba = D.Bin[a];
-  const double* Bc = D.Bin[c];
-  // j_e on the e-edge stored at Y: (B_{c_e}[Y] - B_{c_e}[Y - a_e]) / h_{a_e}
-  //                               - (B_{a_e}[Y] - B_{a_e}[Y - c_e]) / h_{c_e}
-  auto jedge = [&](int e, long long Y) {
-    const int ae = (e + 1) % 3, ce = (e + 2) % 3;
-    const double* Bce = D.Bin[ce];
-    const double* Bae = D.Bin[ae];
-    return fma(Bce[Y] - Bce[shift(D, Y, ae, -1)], D.hinv[ae], -((Bae[Y] - Bae[shift(D, Y, ce, -1)]) * D.hinv[ce]));
-  };
+  const double* Ja = D.Epart + a * D.N;
+  const double* Jc = D.Epart + c * D.N;
+  const double* ba = D.P + (5 + a) * D.N;
+  const double* bc = D.P + (5 + c) * D.N;
   const long long Xc = shift(D, X, c, 1), Xa = shift(D, X, a, 1), Xmd = shift(D, X, d, -1);
-  const double ea = 0.5 * D.eta * (jedge(a, X) + jedge(a, Xc));
-  const double ec = 0.5 * D.eta * (jedge(c, X) + jedge(c, Xa));
-  const double bcbar = 0.25 * (Bc[Xmd] + Bc[X] + Bc[shift(D, Xmd, c, 1)] + Bc[Xc]);
-  const double babar = 0.25 * (Ba[Xmd] + Ba[X] + Ba[shift(D, Xmd, a, 1)] + Ba[Xa]);
-  return fma(ea, bcbar, -ec * babar);
+  const double ea = Ja[X] + Ja[Xc], ec = Jc[X] + Jc[Xa];
+  const double bcbar = halve(bc[Xmd] + bc[X]), babar = halve(ba[Xmd] + ba[X]);
+  return fma(ea, bcbar, -(ec * babar));
 }
 
 // The reconstruction windows of a block's threads in shared memory: slot k of variable v of a

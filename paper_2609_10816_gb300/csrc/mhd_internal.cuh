@@ -25,6 +25,7 @@ struct Dev {
   double dth[3];        // dt / h_d
   const double* dthp;   // when set, dt / h_d are read from device memory here instead (a step whose
                         // dt comes from the device-side CFL reduction)
+  double hcur[3];       // eta / (2 h_d)
   int resistive;        // eta != 0
   int combine;          // stage 2: store (old + new) / 2 into fluxes and EMFs
   int fofc_criteria;    // bit 0 rho <= 0, bit 1 p <= 0
@@ -42,7 +43,9 @@ struct Dev {
   double* Ap;     // [3][N] alpha+ on d-faces
   double* Am;     // [3][N] alpha-
   double* Us;     // [3][N] Q26 face-normal velocity u_d^*
-  double* Epart;  // [3][4][N] per e-edge: b_a^B, b_a^T, u_a^B, u_a^T (reconstructed along c)
+  double* Epart;  // [3][4][N] per e-edge: b_a^B, b_a^T, u_a^B, u_a^T (reconstructed along c); until the
+                  // bottom/top sweep of a stage writes them, [3][N] eta j_e / 2 on the e-edges of the
+                  // stage input (written with its primitives, resistive steps only)
   double* E;      // [3][N] edge EMFs
   // FS18 / B25a extras
   double* VL;     // [3][3][N] FS18: left velocity states on d-faces, component k
@@ -65,6 +68,13 @@ struct Dev {
   unsigned long long* work;
   int stage;      // 0 or 1 (which counter the flux correction reads)
 };
+
+// sets the resistivity and what follows from it (resistive terms are switched by `resistive`)
+inline void set_eta(Dev& D, double eta) {
+  D.eta = eta;
+  D.resistive = eta != 0.0;
+  for (int d = 0; d < 3; ++d) D.hcur[d] = 0.5 * eta * D.hinv[d];
+}
 
 // Work slots of the dynamically scheduled sweeps of one stage.
 constexpr int kWorkSlots = 9;
