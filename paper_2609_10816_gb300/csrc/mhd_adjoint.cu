@@ -867,7 +867,7 @@ __device__ __forceinline__ void prim_rev(const AdjDev& A, long long X, double* l
   const double rho = u[0], rinv = rcp(rho);
   const double ui[3] = {u[1] * rinv, u[2] * rinv, u[3] * rinv};
   const double u2s = fma(ui[0], ui[0], fma(ui[1], ui[1], ui[2] * ui[2]));
-  const double leint = (D.gam - 1.0) * lp[4];        // p = (gamma - 1) eint
+  const double leint = D.gm1 * lp[4];        // p = (gamma - 1) eint
   const double lq = -0.5 * leint;                     // eint = e - (rho u2s + b2s) / 2
   double lrinv = 0.0;
 #pragma unroll
@@ -896,7 +896,7 @@ __global__ void __launch_bounds__(128) k_adj_prim(AdjDev A) {
     // the same quantity for cell X - d (its upper d-face is X's lower one)
     const long long Xm = shift(D, X, d, -1);
     const double bm = 0.5 * (D.Bin[d][Xm] + D.Bin[d][X]);
-    const double lqm = -0.5 * ((D.gam - 1.0) * A.lP[4 * N + Xm]);
+    const double lqm = -0.5 * (D.gm1 * A.lP[4 * N + Xm]);
     const double lbm = fma(2.0 * bm, lqm, A.lP[(5 + d) * N + Xm]);
     A.lB[d * N + X] += 0.5 * (lbc[d] + lbm);
   }
@@ -970,7 +970,7 @@ __device__ __forceinline__ void prim_vjp_atomic(const AdjDev& A, long long Y, co
   const double rho = u[0], rinv = rcp(rho);
   const double ui[3] = {u[1] * rinv, u[2] * rinv, u[3] * rinv};
   const double u2s = fma(ui[0], ui[0], fma(ui[1], ui[1], ui[2] * ui[2]));
-  const double leint = (D.gam - 1.0) * lp[4];  // p = (gamma - 1) eint
+  const double leint = D.gm1 * lp[4];  // p = (gamma - 1) eint
   const double lq = -0.5 * leint;               // eint = e - (rho u2s + b2s) / 2
   double lrinv = 0.0;
 #pragma unroll

@@ -199,7 +199,8 @@ mhd_status mhd_create(const mhd_config* cfg, void* cuda_stream, mhd_ctx** out) {
   D.h[0] = cfg->dx; D.h[1] = cfg->dy; D.h[2] = cfg->dz;
   for (int d = 0; d < 3; ++d) D.hinv[d] = 1.0 / D.h[d];
   D.gam = cfg->gamma;
-  D.gm1inv = 1.0 / (cfg->gamma - 1.0);
+  D.gm1 = cfg->gamma - 1.0;
+  D.gm1inv = 1.0 / D.gm1;
   D.fofc_criteria = cfg->fofc_criteria ? cfg->fofc_criteria : 3;
   // scratch, in doubles per cell: U1 5, B1 3, P 8, F 15, Ap/Am/Us 9, Epart 12, E 3,
   // VL/VR 18, Xpart 24, EfL 6, EfB 6  -> 109; + flags (1 byte) + counters

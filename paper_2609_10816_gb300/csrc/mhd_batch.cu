@@ -261,7 +261,8 @@ mhd_status upload_params(mhd_batch* b, const mhd_batch_state* s, int scheme, dou
     D.stride[0] = 1; D.stride[1] = n[0]; D.stride[2] = (long long)n[0] * n[1];
     for (int d = 0; d < 3; ++d) { D.h[d] = b->h; D.hinv[d] = 1.0 / b->h; }
     D.gam = b->gamma;
-    D.gm1inv = 1.0 / (b->gamma - 1.0);
+    D.gm1 = b->gamma - 1.0;
+    D.gm1inv = 1.0 / D.gm1;
     mhd::set_eta(D, eta);
     D.fofc_criteria = (scheme & MHD_FOFC_OFF) ? 0 : 3;
     D.emf = (scheme >> 8) & 0xf;

@@ -24,7 +24,7 @@ __device__ __forceinline__ void prim_from(const Dev& D, const double* u, const d
   const double b2s = fma(b0, b0, fma(b1, b1, b2 * b2));
   const double eint = u[4] - halve(fma(rho, u2s, b2s));
   w[0] = rho; w[1] = u0; w[2] = u1; w[3] = u2;
-  w[4] = (D.gam - 1.0) * eint;
+  w[4] = D.gm1 * eint;
   w[5] = b0; w[6] = b1; w[7] = b2;
 }
 __device__ __forceinline__ void load_cell(const Dev& D, const double* U, const double* const* B, long long X,
@@ -188,7 +188,7 @@ __device__ __forceinline__ bool invalid_vals(const Dev& D, const double* u, cons
     const double u0 = u[1] * rinv, u1 = u[2] * rinv, u2 = u[3] * rinv;
     const double u2s = fma(u0, u0, fma(u1, u1, u2 * u2));
     const double b2s = fma(bc[0], bc[0], fma(bc[1], bc[1], bc[2] * bc[2]));
-    const double p = (D.gam - 1.0) * (u[4] - halve(fma(rho, u2s, b2s)));
+    const double p = D.gm1 * (u[4] - halve(fma(rho, u2s, b2s)));
     if (!gt0(p)) return true;  // p <= 0 or NaN
   }
   return false;

@@ -20,7 +20,7 @@ struct Dev {
   long long stride[3];  // 1, nx, nx*ny
   double h[3];
   double hinv[3];
-  double gam, gm1inv;
+  double gam, gm1, gm1inv;  // gamma, gamma - 1 and its inverse
   double dt, eta;
   double dth[3];        // dt / h_d
   const double* dthp;   // when set, dt / h_d are read from device memory here instead (a step whose

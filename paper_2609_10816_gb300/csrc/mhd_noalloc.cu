@@ -104,7 +104,8 @@ extern "C" mhd_status mhd_step_noalloc(const mhd_config* cfg, const mhd_state* s
   D.h[0] = cfg->dx; D.h[1] = cfg->dy; D.h[2] = cfg->dz;
   for (int d = 0; d < 3; ++d) D.hinv[d] = 1.0 / D.h[d];
   D.gam = cfg->gamma;
-  D.gm1inv = 1.0 / (cfg->gamma - 1.0);
+  D.gm1 = cfg->gamma - 1.0;
+  D.gm1inv = 1.0 / D.gm1;
   D.fofc_criteria = fofc ? (cfg->fofc_criteria ? cfg->fofc_criteria : 3) : 0;
   D.dt = dt;
   for (int d = 0; d < 3; ++d) D.dth[d] = dt * D.hinv[d];
