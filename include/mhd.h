@@ -132,8 +132,9 @@ enum {
   MHD_K_EDGE_LR = 3,   /* c-face quantities to edges along a + LD04 + eta j, 1 per stage */
   MHD_K_UPDATE = 4,    /* flux divergence and CT update */
   MHD_K_FLAG = 5,      /* validity flags */
-  MHD_K_FOFC = 6,      /* first-order flux correction, 3 launches per stage (exit early if no flag) */
-  MHD_K_MAXSPEED = 7,  /* CFL reduction (and, in mhd_step_cfl, the dt kernel) */
+  MHD_K_FOFC = 6,      /* first-order flux correction, 2 launches per stage (exit early if no flag); the
+                          last one of a step writes S^{n+1} into the caller's arrays */
+  MHD_K_MAXSPEED = 7,  /* CFL reduction (in mhd_step_cfl its last block forms dt) */
   MHD_K_DIVB = 8,      /* divergence reduction */
   MHD_K_EXTRA = 9,     /* scheme-specific extras (FS18 / B25a sweeps) */
   MHD_K_COUNT = 16

@@ -116,7 +116,9 @@ struct Timed {
 // (redone only for cells flux correction changed), or already in place (the CFL reduction)
 enum PrimSource { PRIM_COMPUTE, PRIM_IF_FLAGGED, PRIM_READY };
 
-void run_stage(mhd_ctx* c, const mhd::Dev& D, const Decoded& sc, PrimSource prim = PRIM_COMPUTE) {
+// finish: the stage's result goes into this state's arrays (the last stage), not only into D.Uout.
+void run_stage(mhd_ctx* c, const mhd::Dev& D, const Decoded& sc, PrimSource prim = PRIM_COMPUTE,
+               const mhd_state* finish = nullptr) {
   cudaStream_t st = c->stream;
   if (prim == PRIM_IF_FLAGGED) {
     Timed t(c, MHD_K_PRIM, 1);
@@ -135,7 +137,21 @@ void run_stage(mhd_ctx* c, const mhd::Dev& D, const Decoded& sc, PrimSource prim
   { Timed t(c, MHD_K_EDGE_LR, D.work ? 1 : 3); mhd::launch_edges_lr(D, sc.recon, c->seg, st); }
   { Timed t(c, MHD_K_UPDATE, 1); mhd::launch_update(D, st); }
   { Timed t(c, MHD_K_FLAG, 1); mhd::launch_flag(D, st); }
-  if (sc.fofc) { Timed t(c, MHD_K_FOFC, 3); mhd::launch_fofc(D, st); }
+  if (sc.fofc || finish) {
+    Timed t(c, MHD_K_FOFC, sc.fofc ? 2 : 1);
+    if (sc.fofc) mhd::launch_fofc_fluxes(D, st);
+    if (finish) {
+      double* const b[3] = {finish->b0, finish->b1, finish->b2};
+      mhd::launch_finish(D, sc.fofc, finish->cons, b, st);
+    } else {
+      mhd::launch_fofc_recompute(D, st);
+    }
+  }
+}
+
+// the counters and work cursors of a step, all zero before its first launch
+cudaError_t clear_counters(const mhd::Dev& D, cudaStream_t st) {
+  return cudaMemsetAsync(D.counters, 0, (mhd::kCounters + mhd::kWorkSlots) * sizeof(unsigned long long), st);
 }
 
 }  // namespace
@@ -231,8 +247,8 @@ mhd_status mhd_create(const mhd_config* cfg, void* cuda_stream, mhd_ctx** out) {
   D.Xpart = take(24);
   D.EfL = take(6);
   D.EfB = take(6);
-  D.counters = (unsigned long long*)q;  // 8 counters, then the sweeps' work cursors
-  D.work = D.counters + 8;
+  D.counters = (unsigned long long*)q;  // then the sweeps' work cursors
+  D.work = D.counters + mhd::kCounters;
   c->dtbuf = q + 8 + 16;                  // dt, dt / h_d and an error flag of mhd_step_cfl
   D.flag = (unsigned char*)(q + 8 + 16 + 8);
   e = cudaMemsetAsync(p, 0, bytes, c->stream);
@@ -288,10 +304,10 @@ mhd_status mhd_profile_read(mhd_ctx* ctx, double* total_ms, long long* launches,
   return MHD_OK;
 }
 
-// The two stages and the copy-back of one step; D carries dt / h_d (by value or in device memory).
+// The two stages of one step; D carries dt / h_d (by value or in device memory). prim_ready: the
+// CFL reduction left S^n's primitives (and the counters were cleared before it).
 static mhd_status advance(mhd_ctx* ctx, const mhd_state* state, mhd::Dev D, const Decoded& sc, double eta,
                           bool prim_ready = false) {
-  const long long N = D.N;
   mhd_status s;
   mhd::set_eta(D, eta);
   D.emf = sc.emf;
@@ -299,8 +315,10 @@ static mhd_status advance(mhd_ctx* ctx, const mhd_state* state, mhd::Dev D, cons
   D.U0 = state->cons;
   D.B0[0] = state->b0; D.B0[1] = state->b1; D.B0[2] = state->b2;
   cudaStream_t st = ctx->stream;
-  s = cuda_check(ctx, cudaMemsetAsync(D.counters, 0, 4 * sizeof(unsigned long long), st), "cudaMemsetAsync");
-  if (s != MHD_OK) return s;
+  if (!prim_ready) {
+    s = cuda_check(ctx, clear_counters(D, st), "cudaMemsetAsync");
+    if (s != MHD_OK) return s;
+  }
 
   // stage 1: S^{n+1/2} = S^n + D^n  (Eq. rk1:update), written to scratch
   D.Uin = D.U0;
@@ -319,20 +337,8 @@ static mhd_status advance(mhd_ctx* ctx, const mhd_state* state, mhd::Dev D, cons
   D.combine = 1;
   D.stage = 1;
   D.Pnext = nullptr;
-  run_stage(ctx, D, sc, PRIM_IF_FLAGGED);
-
-  s = cuda_check(ctx, cudaGetLastError(), "kernel launch");
-  if (s != MHD_OK) return s;
-  s = cuda_check(ctx, cudaMemcpyAsync(state->cons, ctx->U1, 5 * N * sizeof(double), cudaMemcpyDeviceToDevice, st),
-                 "cudaMemcpyAsync");
-  if (s != MHD_OK) return s;
-  double* bout[3] = {state->b0, state->b1, state->b2};
-  for (int d = 0; d < 3; ++d) {
-    s = cuda_check(ctx, cudaMemcpyAsync(bout[d], ctx->B1[d], N * sizeof(double), cudaMemcpyDeviceToDevice, st),
-                   "cudaMemcpyAsync");
-    if (s != MHD_OK) return s;
-  }
-  return MHD_OK;
+  run_stage(ctx, D, sc, PRIM_IF_FLAGGED, state);
+  return cuda_check(ctx, cudaGetLastError(), "kernel launch");
 }
 
 mhd_status mhd_step(mhd_ctx* ctx, const mhd_state* state, double dt, int scheme, double eta) {
@@ -359,15 +365,14 @@ mhd_status enqueue_step_cfl(mhd_ctx* ctx, const mhd_state* state, double cfl, co
   mhd::Dev D = ctx->base;
   mhd::set_eta(D, eta);  // (the reduction also leaves the currents of S^n)
   cudaStream_t st = ctx->stream;
-  mhd_status s = cuda_check(ctx, cudaMemsetAsync(D.counters + 2, 0, sizeof(unsigned long long), st),
-                            "cudaMemsetAsync");
+  mhd_status s = cuda_check(ctx, clear_counters(D, st), "cudaMemsetAsync");
   if (s != MHD_OK) return s;
   mhd::Ptr3 B = {{state->b0, state->b1, state->b2}};
   const double hmin = std::fmin(D.h[0], std::fmin(D.h[1], D.h[2]));
   {
-    Timed t(ctx, MHD_K_MAXSPEED, 2);  // the reduction (which also leaves S^n's primitives) and dt
-    mhd::launch_maxspeed(D, state->cons, B, D.counters + 2, st, D.P);
-    mhd::launch_set_dt(D.counters + 2, cfl, eta, hmin, D.hinv, ctx->dtbuf, st);
+    Timed t(ctx, MHD_K_MAXSPEED, 1);  // (it also leaves S^n's primitives)
+    mhd::launch_maxspeed_dt(D, state->cons, B, D.counters + 2,
+                            mhd::DtArgs{cfl, eta, hmin, ctx->dtbuf, D.counters + 4}, st);
   }
   s = cuda_check(ctx, cudaGetLastError(), "kernel launch");
   if (s != MHD_OK) return s;
@@ -609,7 +614,7 @@ mhd_status mhd_step_adjoint(mhd_ctx* ctx, const mhd_state* state, const mhd_stat
   D.combine = 0;
   D.stage = 0;
   const double* lamb[3] = {lam->b0, lam->b1, lam->b2};
-  cudaError_t e = cudaMemsetAsync(D.counters, 0, 4 * sizeof(unsigned long long), st);
+  cudaError_t e = clear_counters(D, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(lamU, lam->cons, 5 * N * sizeof(double), cudaMemcpyDeviceToDevice, st);
   for (int d = 0; d < 3 && e == cudaSuccess; ++d)
     e = cudaMemcpyAsync(lamB + d * N, lamb[d], N * sizeof(double), cudaMemcpyDeviceToDevice, st);
@@ -727,7 +732,7 @@ mhd_status mhd_adjoint_check(mhd_ctx* ctx, long long n, int scheme, unsigned lon
   mhd_status s = decode(ctx, scheme, sc);
   if (s != MHD_OK) return s;
   const mhd::Dev& D = ctx->base;
-  // 7 results: the scratch's work cursors serve (they are rezeroed before every sweep)
+  // 7 results: the scratch's work cursors serve (they are cleared before every step)
   unsigned long long* out = D.work;
   s = cuda_check(ctx, cudaMemsetAsync(out, 0, 7 * sizeof(unsigned long long), ctx->stream), "cudaMemsetAsync");
   if (s != MHD_OK) return s;
@@ -747,7 +752,7 @@ mhd_status mhd_math_check(mhd_ctx* ctx, long long n, double* max_rel_err) {
   ctx->err.clear();
   if (!max_rel_err || n < 1 || n > (1LL << 40)) return fail(ctx, MHD_ERR_ARG, "need 1 <= n <= 2^40 and an output");
   const mhd::Dev& D = ctx->base;
-  // 7 results: the scratch's work cursors serve (they are rezeroed before every sweep)
+  // 7 results: the scratch's work cursors serve (they are cleared before every step)
   unsigned long long* out = D.work;
   mhd_status s = cuda_check(ctx, cudaMemsetAsync(out, 0, 7 * sizeof(unsigned long long), ctx->stream),
                             "cudaMemsetAsync");

@@ -30,35 +30,42 @@ __global__ void __launch_bounds__(256) k_flag(Dev D) {
 }
 // First-order fix-up passes: grid-stride loops over a grid of two waves, so that a stage with
 // no flagged cell (the usual case) costs a few microseconds of early exits
-__global__ void __launch_bounds__(128) k_fo_faces(Dev D) {
+__global__ void __launch_bounds__(128) k_fo_fluxes(Dev D) {
   if (D.counters[D.stage] == 0) return;
-  for (long long X = cell_id(); X < D.N; X += (long long)gridDim.x * blockDim.x) fo_faces_cell(D, X);
-}
-__global__ void __launch_bounds__(128) k_fo_edges(Dev D) {
-  if (D.counters[D.stage] == 0) return;
-  for (long long X = cell_id(); X < D.N; X += (long long)gridDim.x * blockDim.x) fo_edges_cell(D, X);
+  for (long long X = cell_id(); X < D.N; X += (long long)gridDim.x * blockDim.x) {
+    fo_faces_cell(D, X);
+    fo_edges_cell(D, X);
+  }
 }
 __global__ void __launch_bounds__(128) k_fo_recompute(Dev D) {
   if (D.counters[D.stage] == 0) return;
-  for (long long X = cell_id(); X < D.N; X += (long long)gridDim.x * blockDim.x) fo_recompute_cell(D, X);
+  for (long long X = cell_id(); X < D.N; X += (long long)gridDim.x * blockDim.x)
+    fo_recompute_cell(D, X);
 }
-
-// dt = cfl hmin / max(smax, 2 eta / hmin) (Eq. resistivity:cfl), the operations of mhd_max_dt
-__global__ void k_set_dt(const unsigned long long* smax_bits, double cfl, double eta, double hmin, double hx,
-                         double hy, double hz, double* out) {
-  double smax = dfrom((long long)*smax_bits);
-  const double sres = 2.0 * eta / hmin;
-  if (sres > smax) smax = sres;
-  double dt = 0.0, bad = 1.0;
-  if (smax > 0.0 && smax < 1e300) {
-    dt = cfl * hmin / smax;
-    bad = 0.0;
+// The last pass of a step: S^{n+1} into the caller's arrays, the cells and faces that flux
+// correction touches recomputed on the way (from fluxes, EMFs and the cell's own S^n, which those
+// arrays hold until it is written). In the place of a recompute launch and four copies.
+struct Out4 {
+  double* U;
+  double* B[3];
+};
+__global__ void __launch_bounds__(256) k_finish(Dev D, Out4 o, int fofc) {
+  const long long X = cell_id(), N = D.N;
+  if (X >= N) return;
+  double w[8];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) w[v] = D.Uout[v * N + X];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) w[5 + d] = D.Bout[d][X];
+  if (fofc && D.counters[D.stage] == 0) fofc = 0;
+  if (!fofc) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) o.U[v * N + X] = w[v];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) o.B[d][X] = w[5 + d];
+    return;
   }
-  out[0] = dt;
-  out[1] = dt * hx;
-  out[2] = dt * hy;
-  out[3] = dt * hz;
-  out[4] = bad;
+  fo_finish_cell(D, X, w, o.U, o.B);
 }
 
 // ---- reductions -----------------------------------------------------------------------------
@@ -85,10 +92,9 @@ __device__ __forceinline__ void block_max_atomic(double v, unsigned long long* o
   __syncthreads();  // sm[] may be reused by a following call
 }
 
-// max over cells of the CFL signal speed (cfl_speed_max): a grid-stride loop whose warps share
-// their running maximum after every pass, so that most cells are settled by the bound check
-__global__ void __launch_bounds__(256) k_maxspeed(Dev D, const double* U, Ptr3 Bp,
-                                                  unsigned long long* out, double* Pout) {
+// max over a thread's cells of the CFL signal speed (cfl_speed_max): a grid-stride loop whose warps
+// share their running maximum after every pass, so that most cells are settled by the bound check
+__device__ __forceinline__ double cell_speed_max(const Dev& D, const double* U, const Ptr3& Bp, double* Pout) {
   const long long nth = (long long)gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31;
   double s = 0.0;
@@ -101,7 +107,33 @@ __global__ void __launch_bounds__(256) k_maxspeed(Dev D, const double* U, Ptr3 B
     }
     s = __longlong_as_double((long long)b);
   }
-  block_max_atomic(s, out);
+  return s;
+}
+__global__ void __launch_bounds__(256) k_maxspeed(Dev D, const double* U, Ptr3 Bp, unsigned long long* out) {
+  block_max_atomic(cell_speed_max(D, U, Bp, nullptr), out);
+}
+
+// The same reduction, with S^n's primitives, and dt by the last block to finish (the operations of
+// mhd_max_dt): dt = cfl hmin / max(smax, 2 eta / hmin) (Eq. resistivity:cfl)
+__device__ __forceinline__ void set_dt(const Dev& D, const DtArgs& a, double smax) {
+  const double sres = 2.0 * a.eta / a.hmin;
+  if (sres > smax) smax = sres;
+  double dt = 0.0, bad = 1.0;
+  if (smax > 0.0 && smax < 1e300) {
+    dt = a.cfl * a.hmin / smax;
+    bad = 0.0;
+  }
+  a.out[0] = dt;
+  for (int d = 0; d < 3; ++d) a.out[1 + d] = dt * D.hinv[d];
+  a.out[4] = bad;
+}
+__global__ void __launch_bounds__(256) k_maxspeed_dt(Dev D, const double* U, Ptr3 Bp, unsigned long long* smax,
+                                                     DtArgs a) {
+  block_max_atomic(cell_speed_max(D, U, Bp, D.P), smax);
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(a.done, 1ull) == gridDim.x - 1) set_dt(D, a, dfrom((long long)atomicMax(smax, 0ull)));
+  }
 }
 
 // max over cells of |div b| and over faces of |b|
@@ -252,22 +284,24 @@ void launch_flag(const Dev& d, cudaStream_t st) { k_flag<<<blocks_for(d.N, 256),
 void launch_prim_if_flagged(const Dev& d, int prev_stage, cudaStream_t st) {
   k_prim_if_flagged<<<blocks_for(d.N, 256), 256, 0, st>>>(d, prev_stage);
 }
-void launch_set_dt(const unsigned long long* smax_bits, double cfl, double eta, double hmin, const double* hinv,
-                   double* out, cudaStream_t st) {
-  k_set_dt<<<1, 1, 0, st>>>(smax_bits, cfl, eta, hmin, hinv[0], hinv[1], hinv[2], out);
+static unsigned two_waves(const void* k, int bs, long long n) {
+  return (unsigned)std::min((long long)blocks_for(n, bs), 2LL * resident_blocks(k, bs));
 }
-void launch_fofc(const Dev& d, cudaStream_t st) {
-  auto grid = [&](const void* k) {
-    return (unsigned)std::min((long long)blocks_for(d.N, 128), 2LL * resident_blocks(k, 128));
-  };
-  k_fo_faces<<<grid((const void*)k_fo_faces), 128, 0, st>>>(d);
-  k_fo_edges<<<grid((const void*)k_fo_edges), 128, 0, st>>>(d);
-  k_fo_recompute<<<grid((const void*)k_fo_recompute), 128, 0, st>>>(d);
+void launch_fofc_fluxes(const Dev& d, cudaStream_t st) {
+  k_fo_fluxes<<<two_waves((const void*)k_fo_fluxes, 128, d.N), 128, 0, st>>>(d);
 }
-void launch_maxspeed(const Dev& d, const double* U, Ptr3 B, unsigned long long* out, cudaStream_t st,
-                     double* Pout) {
-  const long long cap = 2LL * resident_blocks((const void*)k_maxspeed, 256);  // two waves of blocks
-  k_maxspeed<<<(unsigned)std::min((long long)blocks_for(d.N, 256), cap), 256, 0, st>>>(d, U, B, out, Pout);
+void launch_fofc_recompute(const Dev& d, cudaStream_t st) {
+  k_fo_recompute<<<two_waves((const void*)k_fo_recompute, 128, d.N), 128, 0, st>>>(d);
+}
+void launch_finish(const Dev& d, bool fofc, double* U, double* const* B, cudaStream_t st) {
+  k_finish<<<blocks_for(d.N, 256), 256, 0, st>>>(d, Out4{U, {B[0], B[1], B[2]}}, fofc ? 1 : 0);
+}
+void launch_maxspeed(const Dev& d, const double* U, Ptr3 B, unsigned long long* out, cudaStream_t st) {
+  k_maxspeed<<<two_waves((const void*)k_maxspeed, 256, d.N), 256, 0, st>>>(d, U, B, out);
+}
+void launch_maxspeed_dt(const Dev& d, const double* U, Ptr3 B, unsigned long long* smax, const DtArgs& a,
+                        cudaStream_t st) {
+  k_maxspeed_dt<<<two_waves((const void*)k_maxspeed_dt, 256, d.N), 256, 0, st>>>(d, U, B, smax, a);
 }
 void launch_divb(const Dev& d, Ptr3 B, unsigned long long* out, cudaStream_t st) {
   k_divb<<<blocks_for(d.N, 256), 256, 0, st>>>(d, B, out);

@@ -347,15 +347,12 @@ __device__ __forceinline__ void fo_edges_cell(const Dev& D, long long X) {
   }
 }
 
-// Recompute every cell with a masked face and every face with a masked edge.
-__device__ __forceinline__ void fo_recompute_cell(const Dev& D, long long X) {
-  const long long N = D.N;
-  const long long Xp[3] = {shift(D, X, 0, 1), shift(D, X, 1, 1), shift(D, X, 2, 1)};
+// Every cell with a masked face and every face with a masked edge is recomputed. cell: whether X is
+// such a cell, face[d]: whether its lower d-face is such a face; Xp: X + 1 along each axis.
+__device__ __forceinline__ void fo_touched(const Dev& D, long long X, const long long* Xp, bool& cell, bool* face) {
   const long long Xm[3] = {shift(D, X, 0, -1), shift(D, X, 1, -1), shift(D, X, 2, -1)};
-  bool cell = flagged(D, X);
+  cell = flagged(D, X);
   for (int d = 0; d < 3; ++d) cell = cell || flagged(D, Xp[d]) || flagged(D, Xm[d]);
-  if (cell)
-    for (int v = 0; v < 5; ++v) D.Uout[v * N + X] = cell_new(D, v, X, Xp);
   // e-edge at Y is masked if one of Y, Y-a, Y-c, Y-a-c is flagged
   auto edge_masked = [&](int e, long long Y) {
     const int a = (e + 1) % 3, c = (e + 2) % 3;
@@ -365,9 +362,27 @@ __device__ __forceinline__ void fo_recompute_cell(const Dev& D, long long X) {
   for (int d = 0; d < 3; ++d) {
     const int a = (d + 1) % 3, c = (d + 2) % 3;
     // the d-face at X is bounded by c-edges at X and X+a, and a-edges at X and X+c
-    if (edge_masked(c, X) || edge_masked(c, Xp[a]) || edge_masked(a, X) || edge_masked(a, Xp[c]))
-      D.Bout[d][X] = face_new(D, d, X, Xp);
+    face[d] = edge_masked(c, X) || edge_masked(c, Xp[a]) || edge_masked(a, X) || edge_masked(a, Xp[c]);
   }
+}
+__device__ __forceinline__ void fo_recompute_cell(const Dev& D, long long X) {
+  const long long Xp[3] = {shift(D, X, 0, 1), shift(D, X, 1, 1), shift(D, X, 2, 1)};
+  bool cell, face[3];
+  fo_touched(D, X, Xp, cell, face);
+  if (cell)
+    for (int v = 0; v < 5; ++v) D.Uout[v * D.N + X] = cell_new(D, v, X, Xp);
+  for (int d = 0; d < 3; ++d)
+    if (face[d]) D.Bout[d][X] = face_new(D, d, X, Xp);
+}
+// cell X of the step's result into U, B: w (5 conserved values, 3 lower faces), recomputed where
+// touched. U, B may be the arrays of S^n: only the cell's own values of it are read.
+__device__ __forceinline__ void fo_finish_cell(const Dev& D, long long X, const double* w, double* U,
+                                               double* const* B) {
+  const long long Xp[3] = {shift(D, X, 0, 1), shift(D, X, 1, 1), shift(D, X, 2, 1)};
+  bool cell, face[3];
+  fo_touched(D, X, Xp, cell, face);
+  for (int v = 0; v < 5; ++v) U[v * D.N + X] = cell ? cell_new(D, v, X, Xp) : w[v];
+  for (int d = 0; d < 3; ++d) B[d][X] = face[d] ? face_new(D, d, X, Xp) : w[5 + d];
 }
 
 }  // namespace mhd

@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(128) k_edges(Dev D, int s0, int s1, int s2) {
   long long tot[3];
 #pragma unroll
   for (int e = 0; e < 3; ++e) tot[e] = sweep_threads(D, LR ? (e + 1) % 3 : (e + 2) % 3, sg[e]);
-  for_each_segment(D.work + (LR ? 6 : 3), tot[0] + tot[1] + tot[2], [&](long long t) {
+  for_each_segment(work_cursor(D, LR ? CUR_EDGE_LR : CUR_EDGE_BT), tot[0] + tot[1] + tot[2], [&](long long t) {
     int e = 0;
     if (t >= tot[0]) {
       t -= tot[0];
@@ -76,7 +76,6 @@ static void launch_edges_t(const Dev& d, int seg, cudaStream_t st) {
     tot += sweep_threads(d, dir, sg[e]);
   }
   const long long blocks = std::min((tot + bs - 1) / bs, res);
-  cudaMemsetAsync(d.work + (LR ? 6 : 3), 0, sizeof(unsigned long long), st);
   k_edges<RC, EMF, LR><<<(unsigned)blocks, bs, 0, st>>>(d, sg[0], sg[1], sg[2]);
 }
 

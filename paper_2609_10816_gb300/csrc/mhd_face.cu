@@ -26,7 +26,7 @@ template <int RC, int RS>
 __global__ void __launch_bounds__(kFaceThreads, kFaceMinBlocks) k_faces(Dev D, int s0, int s1, int s2, int x_lanes) {
   const long long t0 = x_lanes ? lane_threads(D, 0, s0) : round32(sweep_threads(D, 0, s0));
   const long long t1 = round32(sweep_threads(D, 1, s1)), t2 = round32(sweep_threads(D, 2, s2));
-  for_each_segment(D.work, t0 + t1 + t2, [&](long long t) {
+  for_each_segment(work_cursor(D, CUR_FACE), t0 + t1 + t2, [&](long long t) {
     int dir = 0, seg = s0;
     if (t >= t0) {
       t -= t0;
@@ -61,11 +61,16 @@ static void launch_faces_t(const Dev& d, int seg, cudaStream_t st) {
       tot += lane_threads(d, dir, sg[dir]);
     } else {
       sg[dir] = fill_seg(d, dir, seg, res * bs);
+      // a face in a walk waits for the one before it (about 7 us each on an idle GPU), so boxes that
+      // leave it idle walk 2 faces, and the smallest one, though each walk starts its windows anew
+      // (face sweeps of a PPM + HLLD step with 4, 2 and 1: 8^3 104, 67, 48 us; 24^3 108, 88, 74;
+      // 32^3 144, 112, 128; 48^3 324, 292, 332)
+      if (sg[dir] <= 4 && sweep_threads(d, dir, 2) <= res * bs) sg[dir] = 2;
+      if (sg[dir] <= 2 && 3 * sweep_threads(d, dir, 1) <= res * bs) sg[dir] = 1;
       tot += sweep_threads(d, dir, sg[dir]) + 31;
     }
   }
   const long long blocks = std::min((tot + bs - 1) / bs, res);
-  cudaMemsetAsync(d.work, 0, sizeof(unsigned long long), st);
   k_faces<RC, RS><<<(unsigned)blocks, bs, smem, st>>>(d, sg[0], sg[1], sg[2], x_lanes ? 1 : 0);
 }
 

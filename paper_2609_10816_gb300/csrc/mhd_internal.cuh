@@ -63,8 +63,8 @@ struct Dev {
                   // four c-face velocity states, [3][10][N]; B25a b_c and the two c-face EMF
                   // values, in the first 6 of [3][10][N]
   unsigned long long* counters;  // [0] stage-1 flagged cells, [1] stage-2, [2..3] reductions
-  // work-list cursors of the dynamically scheduled sweeps ([dir] face, [3 + e] edge_bt,
-  // [6 + e] edge_lr), zeroed before every stage; NULL: one segment per thread, no cursor
+  // work-list cursors of the dynamically scheduled sweeps (work_cursor), zero before every step;
+  // NULL: one segment per thread, no cursor
   unsigned long long* work;
   int stage;      // 0 or 1 (which counter the flux correction reads)
 };
@@ -76,8 +76,14 @@ inline void set_eta(Dev& D, double eta) {
   for (int d = 0; d < 3; ++d) D.hcur[d] = 0.5 * eta * D.hinv[d];
 }
 
-// Work slots of the dynamically scheduled sweeps of one stage.
-constexpr int kWorkSlots = 9;
+// Counters and cursors of a context: 8 counters, then 8 cursors, cleared by one memset per step.
+constexpr int kCounters = 8;
+constexpr int kWorkSlots = 8;
+enum { CUR_FACE = 0, CUR_EDGE_BT = 1, CUR_EDGE_LR = 2 };
+// the cursor of one sweep launch (each has its own per stage, so that they need no clearing between)
+__host__ __device__ inline unsigned long long* work_cursor(const Dev& D, int sweep) {
+  return D.work + 4 * D.stage + sweep;
+}
 
 // Adjoint of the flux function at a stage input state (mhd_adjoint.cu).
 struct AdjDev {
@@ -130,15 +136,24 @@ void launch_edges_bt(const Dev& d, int recon, int seg, cudaStream_t st);
 void launch_edges_lr(const Dev& d, int recon, int seg, cudaStream_t st);
 void launch_update(const Dev& d, cudaStream_t st);
 void launch_flag(const Dev& d, cudaStream_t st);
-// dt of Eq. (resistivity:cfl) from the reduction's maximum signal speed (bit pattern at smax_bits):
-// out[0] = dt, out[1..3] = dt / h_d, out[4] = 1 when the speed is zero or not finite (dt = 0)
-void launch_set_dt(const unsigned long long* smax_bits, double cfl, double eta, double hmin, const double* hinv,
-                   double* out, cudaStream_t st);
 void launch_prim_if_flagged(const Dev& d, int prev_stage, cudaStream_t st);
-void launch_fofc(const Dev& d, cudaStream_t st);
-// Pout (may be NULL): the primitives of U, B written as the reduction forms them
-void launch_maxspeed(const Dev& d, const double* U, Ptr3 B, unsigned long long* out, cudaStream_t st,
-                     double* Pout = nullptr);
+// first-order fluxes and EMFs of the flagged cells' faces and edges
+void launch_fofc_fluxes(const Dev& d, cudaStream_t st);
+// the touched cells and faces recomputed in d.Uout, d.Bout
+void launch_fofc_recompute(const Dev& d, cudaStream_t st);
+// the stage's result d.Uout, d.Bout, with the touched cells and faces recomputed (fofc), into U, B
+void launch_finish(const Dev& d, bool fofc, double* U, double* const* B, cudaStream_t st);
+void launch_maxspeed(const Dev& d, const double* U, Ptr3 B, unsigned long long* out, cudaStream_t st);
+// the reduction with the primitives in d.P, and by its last block (`done`: a counter that is zero
+// before) dt of Eq. (resistivity:cfl) from the maximum signal speed: out[0] = dt, out[1..3] = dt / h_d,
+// out[4] = 1 when the speed is zero or not finite (dt = 0)
+struct DtArgs {
+  double cfl, eta, hmin;
+  double* out;
+  unsigned long long* done;
+};
+void launch_maxspeed_dt(const Dev& d, const double* U, Ptr3 B, unsigned long long* smax, const DtArgs& a,
+                        cudaStream_t st);
 void launch_divb(const Dev& d, Ptr3 B, unsigned long long* out, cudaStream_t st);
 void launch_math_check(long long n, unsigned long long* out, cudaStream_t st);
 

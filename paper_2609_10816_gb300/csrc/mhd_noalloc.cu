@@ -153,14 +153,15 @@ extern "C" mhd_status mhd_step_noalloc(const mhd_config* cfg, const mhd_state* s
     mhd::launch_edges_lr(D, recon, seg, st);
     mhd::launch_update(D, st);
     mhd::launch_flag(D, st);
-    if (fofc) mhd::launch_fofc(D, st);
+    if (fofc) mhd::launch_fofc_fluxes(D, st);
+    if (stage == 1) {
+      double* const b[3] = {state->b0, state->b1, state->b2};
+      mhd::launch_finish(D, fofc, state->cons, b, st);
+    } else if (fofc) {
+      mhd::launch_fofc_recompute(D, st);
+    }
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(MHD_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
-  e = cudaMemcpyAsync(state->cons, U1, 5 * N * sizeof(double), cudaMemcpyDeviceToDevice, st);
-  double* bout[3] = {state->b0, state->b1, state->b2};
-  for (int d = 0; d < 3 && e == cudaSuccess; ++d)
-    e = cudaMemcpyAsync(bout[d], B1[d], N * sizeof(double), cudaMemcpyDeviceToDevice, st);
-  if (e != cudaSuccess) return fail(MHD_ERR_CUDA, std::string("cudaMemcpyAsync: ") + cudaGetErrorString(e));
   return MHD_OK;
 }
