@@ -491,20 +491,18 @@ struct RevPPM {
   // lam_lo, lam_hi: adjoints of point i's lower / upper values; qn = q_{i+3}. Returns the adjoint of
   // q_{i-2}.
   __device__ __forceinline__ double step(double lam_lo, double lam_hi, double qn) {
-    double lL = lam_lo, lR = lam_hi, gi = 0.0;
+    // FLAT: aL = aR = q_i; FIX_L: aL = 3 q_i - 2 aR; FIX_R: aR = 3 q_i - 2 aL. With x the adjoint of
+    // the fixed value (FLAT: of the lower one) and y of the other, q_i gets 3 x (x + y) and the other
+    // interface y - 2 x (nothing), formed by every lane in two instructions: short branches would be
+    // predicated, and a predicated-off FP64 instruction takes the pipe all the same.
     const int mc = ppm_mono_case(s1, s2);
-    if (mc == PPM_FLAT) {  // aL = aR = q_i
-      gi = lam_lo + lam_hi;
-      lL = lR = 0.0;
-    } else if (mc == PPM_FIX_L) {  // aL = 3 q_i - 2 aR
-      gi = 3.0 * lam_lo;
-      lR = fma(-2.0, lam_lo, lam_hi);
-      lL = 0.0;
-    } else if (mc == PPM_FIX_R) {  // aR = 3 q_i - 2 aL
-      gi = 3.0 * lam_hi;
-      lL = fma(-2.0, lam_hi, lam_lo);
-      lR = 0.0;
-    }
+    const bool fix = mc == PPM_FIX_L || mc == PPM_FIX_R;
+    const double x = mc == PPM_FIX_R ? lam_hi : lam_lo, y = mc == PPM_FIX_R ? lam_lo : lam_hi;
+    const double g3 = fma(fix ? 3.0 : 1.0, x, mc == PPM_FLAT ? y : 0.0);
+    const double gi = mc == PPM_KEEP ? 0.0 : g3;
+    const double o = fma(-2.0, x, y);
+    const double lL = mc == PPM_KEEP ? lam_lo : (mc == PPM_FIX_R ? o : 0.0);
+    const double lR = mc == PPM_KEEP ? lam_hi : (mc == PPM_FIX_L ? o : 0.0);
     const double lf = lfp + lL;           // f_{i-1/2}, complete
     g1 += lf;                             // its q_{i-1}
     double le1 = halve(lf);               // its e_{i-1}
@@ -679,9 +677,16 @@ __device__ __forceinline__ void riemann_grad_rev(const double* WL, const double*
   g[14] = dbn;
 }
 
+// Bound by the FP64 pipe. 3 blocks per SM cost a few spills at 168 registers and are still the faster
+// form (64^3 step 3.79 ms against 3.81 with 2 blocks). The side-based reverse sweep, which doubles
+// nothing for the two choices of side and reverses the wave speed of one side only, took it from
+// 4.13 ms.
+constexpr int kAdjFaceMinBlocks = 3;
+// (the three directions in one launch, blockIdx.y: one tail instead of three)
 template <int RC, int RS>
-__global__ void __launch_bounds__(128) k_adj_faces(AdjDev A, int dir) {
+__global__ void __launch_bounds__(128, kAdjFaceMinBlocks) k_adj_faces(AdjDev A) {
   const Dev& D = A.D;
+  const int dir = blockIdx.y;
   const long long t = aid();
   if (t >= D.N) return;
   const long long f = tiled_cell(D, t);  // a warp's faces on an 8 x 4 patch: fewer divergent fan branches
@@ -822,8 +827,9 @@ __device__ __forceinline__ double joule_adj(const AdjDev& A, int d, long long X,
 }
 
 
-__global__ void __launch_bounds__(128) k_adj_joule(AdjDev A, int d) {
+__global__ void __launch_bounds__(128) k_adj_joule(AdjDev A) {
   const Dev& D = A.D;
+  const int d = blockIdx.y;
   if (!D.resistive) return;
   const long long X = aid();
   const long long N = D.N;
@@ -1155,7 +1161,12 @@ template <int KIND, int EMF = EMF_Q26>
 static void rec_sweeps(const AdjDev& A, cudaStream_t st) {
   const int nsrc = KIND == 1 ? 7 : (KIND == 2 ? 2 : (EMF == EMF_FS18 ? 10 : (EMF == EMF_B25A ? 6 : 4)));
   for (int s = 0; s < 3; ++s) {
-    const int seg = 32;
+    // a segment of seg points takes seg + 4 steps, one after the other (about 2 us each on an idle
+    // GPU): halved, down to 4, until half the threads that fit have work (32^3 step with segments
+    // of 32 points 1.55 ms, so 0.99)
+    int seg = 32;
+    const long long res = 128LL * resident_blocks((const void*)k_adj_rec_sweep<KIND, EMF>, 128);
+    while (seg > 4 && sweep_threads(A.D, s, seg) * nsrc < res / 2) seg /= 2;
     const long long n = sweep_threads(A.D, s, seg) * nsrc;
     k_adj_rec_sweep<KIND, EMF><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(A, s, seg);
   }
@@ -1232,12 +1243,11 @@ static void adj_flux_r(const AdjDev& A, int rs, cudaStream_t st) {
   if (A.D.emf == EMF_FS18) adj_edges_t<RC, EMF_FS18>(A, st);
   else if (A.D.emf == EMF_B25A) adj_edges_t<RC, EMF_B25A>(A, st);
   else adj_edges_t<RC, EMF_Q26>(A, st);
-  for (int dir = 0; dir < 3; ++dir) {
-    if (rs == RS_HLL) k_adj_faces<RC, RS_HLL><<<nb, 128, 0, st>>>(A, dir);
-    else if (rs == RS_HLLD) k_adj_faces<RC, RS_HLLD><<<nb, 128, 0, st>>>(A, dir);
-    else k_adj_faces<RC, RS_LLF><<<nb, 128, 0, st>>>(A, dir);
-    if (A.D.resistive) k_adj_joule<<<nb, 128, 0, st>>>(A, dir);
-  }
+  const dim3 nb3(nb, 3);
+  if (rs == RS_HLL) k_adj_faces<RC, RS_HLL><<<nb3, 128, 0, st>>>(A);
+  else if (rs == RS_HLLD) k_adj_faces<RC, RS_HLLD><<<nb3, 128, 0, st>>>(A);
+  else k_adj_faces<RC, RS_LLF><<<nb3, 128, 0, st>>>(A);
+  if (A.D.resistive) k_adj_joule<<<nb3, 128, 0, st>>>(A);
   if (RC == REC_PPM) rec_sweeps<1>(A, st);
   else k_adj_face_rec<RC><<<nb, 128, 0, st>>>(A);
   k_adj_prim<<<nb, 128, 0, st>>>(A);

@@ -742,6 +742,11 @@ template <class T> struct PhysFluxT {
 };
 using PhysFlux = PhysFluxT<double>;
 
+// a + b with no product fused into it: the larger-speed decision (fast_left) compares the two sides,
+// and equal states have to tie however the code around them is compiled
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ Dual add_rn(Dual a, Dual b) { return Dual(__dadd_rn(a.v, b.v), a.t + b.t); }
+
 // Total pressure and the fast magnetosonic speed of Eq. (waves:fast-speed) along the normal, as
 // A = 2 rho c_f^2 = P + b^2 + sqrt((P + b^2)^2 - 4 P b_n^2) with P = gamma p: neither the
 // discriminant nor A needs 1/rho.
@@ -751,7 +756,7 @@ __device__ __forceinline__ void phys_speed_a(const FaceStateT<T>& s, T bn2, doub
   o.b2 = b2;
   o.pt = s.p + halve(b2);
   const T P = gam * s.p;
-  const T Sp = P + b2;
+  const T Sp = add_rn(P, b2);
   T disc = fma(Sp, Sp, -(times4(bn2) * P));  // 4 bn^2 exactly, on the integer pipe
   disc = pmax(disc, T(0.0));
   o.A = Sp + sqrt_(disc);

@@ -14,38 +14,32 @@
 
 namespace mhd {
 
-// adjoint of phys_speed (b2, pt, cf2 of a state): accumulates into ds and dbn
-__device__ __forceinline__ void phys_speed_rev(const FaceState& s, double bn, double gam, double db2, double dpt,
-                                               double dcf2, FaceState& ds, double& dbn) {
-  const double bn2 = bn * bn;
-  const double b2 = fma(s.by, s.by, fma(s.bz, s.bz, bn2));
+// adjoint of cf2 = A / (2 rho) of a state (phys_speed): accumulates into ds (rho and p) and dbn2, and
+// returns the adjoint of its b2
+__device__ __forceinline__ double speed_rev(const FaceState& s, double bn2, double b2, double A, double gam,
+                                            double dcf2, FaceState& ds, double& dbn2) {
   const double P = gam * s.p;
   const double Sp = P + b2;
-  const double disc0 = fma(Sp, Sp, (-4.0 * bn2) * P);
-  const bool keep = dbits(disc0) >= dbits(0.0);  // pmax(disc, 0) keeps disc
-  const double disc = keep ? disc0 : 0.0;
-  const double q1 = rsqrt_(disc);
-  const double sd = is_zero(disc) ? 0.0 : disc * q1;
+  const double disc0 = fma(Sp, Sp, -(times4(bn2) * P));
+  const bool keep = gt0(disc0);  // (pmax(disc, 0); the square root's derivative at 0 is taken as 0)
   const double r = rcp(s.rho);
-  // cf2 = (r / 2) (Sp + sd)
-  const double dh = dcf2 * (Sp + sd);
-  double dSp = dcf2 * 0.5 * r;
-  const double dsd = dSp;
-  ds.rho -= 0.5 * dh * r * r;
-  // sd = sqrt(disc): derivative rsqrt / 2, taken as 0 at 0
-  const double ddisc = (keep && !is_zero(disc)) ? 0.5 * q1 * dsd : 0.0;
-  // disc = Sp^2 - 4 bn2 P
-  dSp += 2.0 * Sp * ddisc;
-  double dbn2 = -4.0 * P * ddisc;
-  const double dP = -4.0 * bn2 * ddisc + dSp;  // Sp = P + b2
-  double db2t = db2 + dSp;
-  ds.p += gam * dP;
+  double dSp = halve(dcf2) * r;  // A = Sp + sqrt(disc)
+  ds.rho -= dSp * A * r;
+  const double q = halve(rsqrt_(keep ? disc0 : 1.0)) * dSp;
+  const double ddisc = keep ? q : 0.0;
+  dSp = fma(2.0 * Sp, ddisc, dSp);
+  const double d4 = -4.0 * ddisc;
+  dbn2 = fma(P, d4, dbn2);
+  ds.p = fma(gam, fma(bn2, d4, dSp), ds.p);
+  return dSp;
+}
+// adjoint of b2 and pt of a state: accumulates into ds and dbn2
+__device__ __forceinline__ void pt_rev(const FaceState& s, double db2, double dpt, FaceState& ds, double& dbn2) {
+  const double t = fma(0.5, dpt, db2);
   ds.p += dpt;
-  db2t += 0.5 * dpt;
-  ds.by += 2.0 * s.by * db2t;
-  ds.bz += 2.0 * s.bz * db2t;
-  dbn2 += db2t;
-  dbn += 2.0 * bn * dbn2;
+  ds.by = fma(2.0 * s.by, t, ds.by);
+  ds.bz = fma(2.0 * s.bz, t, ds.bz);
+  dbn2 += t;
 }
 
 // adjoint of phys_flux (U, F, e of a state, given its b2 and pt): dU, dF, de in; accumulates
@@ -132,27 +126,19 @@ __device__ __forceinline__ void star_state_rev(const FaceState& q, double m, dou
   dbn2 -= dnum + dden;
 }
 
-__device__ __forceinline__ void add_side(bool left, FaceState& dl, FaceState& dr, const FaceState& d) {
-  FaceState& t = left ? dl : dr;
-  t.rho += d.rho;
-  t.u += d.u;
-  t.v += d.v;
-  t.w += d.w;
-  t.p += d.p;
-  t.by += d.by;
-  t.bz += d.bz;
-}
-
-// Reverse sweep of hlld(): dF in; accumulates into dsl, dsr, dbn, the adjoints of the two sides'
-// b2 / pt (dLb2, dLpt, dRb2, dRpt) and of SL, SR. Like hlld it has one flux formula, that of the
-// state at x/t = 0, whose reverse all lanes take together; inside the fan the reverse of the
-// double-star and star states follows. Against transposing the flux differences across the waves
-// this is about a third fewer FP64 instructions (the 64^3 adjoint step 5.03 ms against 5.76).
+// Reverse sweep of hlld(), in terms of the side `a` whose state the face takes and the other side
+// `o` (left: a is the left one), so that no operation is doubled for the two choices: with
+// du = u_o - u_a and dp = pt_a - pt_o, S_M = u_a + d and d = (m_o du + dp) / (m_o - m_a) for both.
+// Like hlld it has one flux formula, that of the state at x/t = 0, whose reverse all lanes take
+// together; inside the fan the reverse of the double-star and star states follows.
+struct HlldAdj {
+  bool left;
+  FaceState qa, qo;             // adjoints of the two states (o: 0 outside the fan)
+  double pta, pto, b2a, Sa, So;  // of pt, b2 and the outer wave speeds
+};
 __device__ __forceinline__ void hlld_rev(const FaceState& sl, const FaceState& sr, double bn, double bn2,
                                          double gm1inv, const PhysFlux& L, const PhysFlux& R, double SL, double SR,
-                                         const double* dF, FaceState& dsl, FaceState& dsr, double& dbn,
-                                         double& dLb2, double& dLpt, double& dRb2, double& dRpt, double& dSL,
-                                         double& dSR) {
+                                         const double* dF, HlldAdj& G, double& dbn, double& dbn2) {
   // ---- forward values (as in hlld) ----
   const bool supL = gt0(SL);
   const bool fan = !supL && !lt0(SR);
@@ -234,18 +220,18 @@ __device__ __forceinline__ void hlld_rev(const FaceState& sl, const FaceState& s
   double drho = dmu * un;
   double dun = fma(dmu, rho, fma(dF[1], mu, dF[4] * (e + pt)));
   double dP = fma(dF[4], un, dF[1]);
-  double dbn2 = -dF[1];
+  dbn2 -= dF[1];
   double dv = dF[2] * mu, dw = dF[3] * mu;
   dbn -= fma(dF[2], by, fma(dF[3], bz, dF[4] * ub));
   double dby = -(dF[2] * bn), dbz = -(dF[3] * bn);
   double de = dF[4] * un, dub = -(dF[4] * bn);
-  FaceState dq = {0, 0, 0, 0, 0, 0, 0};
+  FaceState dq = {0, 0, 0, 0, 0, 0, 0}, dqo = {0, 0, 0, 0, 0, 0, 0};
   double dqpt = dP;
+  G.pto = G.Sa = G.So = 0.0;
   if (fan) {
     // so far dP is the adjoint of p_t*, dun that of S_M, drho that of rho_a*
     double dSM = dun, dvbs = dub, dsu = 0.0, dm = 0.0, dd = 0.0, dssm = 0.0;
     StarAdj da = {drho, dv, dw, dby, dbz};
-    FaceState dqo = {0, 0, 0, 0, 0, 0, 0};
     double dmo = 0.0, dsuo = 0.0;
     if (dstar) {
       // e = es + ssq (ub - vbs)
@@ -303,45 +289,27 @@ __device__ __forceinline__ void hlld_rev(const FaceState& sl, const FaceState& s
     da.ws = fma(dvbs, a.bzs, da.ws);
     da.bzs = fma(dvbs, a.ws, da.bzs);
     star_state_rev(q, m, su, d, ssm, bn, bn2, ssminv, a, da, es, des, dq, dm, dsu, dd, dssm, dbn, dbn2);
-    // ssm = su - d, p_t* = pt + m d, d = nS dinv, S_M = nL dinv + u_L
+    // ssm = su - d, p_t* = pt + m d, S_M = u_a + d
     dsu += dssm;
-    dd = fma(dP, m, dd - dssm);
+    dd = fma(dP, m, dd - dssm) + dSM;
     dm = fma(dP, d, dm);
     dqpt += dP;
-    const double dnS = dd * dinv;
-    double dnL = dSM * dinv;
-    const double ddinv = fma(dnS, nS, dnL * nL);  // (times dinv)
-    dsl.u += dSM;
-    double dmL = left ? dm : dmo, dmR = left ? dmo : dm;
-    double ddu = 0.0, ddpt = dnS;
-    if (left) {
-      dnL += dnS;
-      ddpt = 0.0;
-    } else {  // nS = mL du + dpt
-      dmL = fma(dnS, du, dmL);
-      ddu = dnS * mL;
-    }
-    // nL = mR du + dpt
-    dmR = fma(dnL, du, dmR);
-    ddu = fma(dnL, mR, ddu);
-    ddpt += dnL;
-    // dinv = 1 / (mR - mL)
-    const double dD = -(ddinv * dinv);
-    dmR += dD;
-    dmL -= dD;
-    dsr.u += ddu;
-    dsl.u -= ddu;
-    dLpt += ddpt;
-    dRpt -= ddpt;
-    // mL = suL rhoL, suL = SL - uL (and R)
-    const double dsuL = fma(dmL, sl.rho, left ? dsu : dsuo), dsuR = fma(dmR, sr.rho, left ? dsuo : dsu);
-    dsl.rho = fma(dmL, suL, dsl.rho);
-    dsr.rho = fma(dmR, suR, dsr.rho);
-    dSL += dsuL;
-    dsl.u -= dsuL;
-    dSR += dsuR;
-    dsr.u -= dsuR;
-    if (dstar) add_side(!left, dsl, dsr, dqo);
+    // d = (m_o du + dp) / (m_o - m_a)
+    const double dn = dd * (left ? dinv : neg_if(true, dinv)), dD = dn * d;
+    const double mot = left ? mR : mL, suot = left ? suR : suL;
+    const FaceState qt = pick(!left, sl, sr);
+    dmo += fma(dn, left ? du : neg_if(true, du), -dD);
+    dm += dD;
+    const double ddu = dn * mot;
+    dqpt += dn;
+    G.pto = -dn;
+    // m = su rho, su = S - u on both sides
+    G.Sa = fma(dm, q.rho, dsu);
+    dq.rho = fma(dm, su, dq.rho);
+    dq.u += dSM - ddu - G.Sa;
+    G.So = fma(dmo, qt.rho, dsuo);
+    dqo.rho = fma(dmo, suot, dqo.rho);
+    dqo.u += ddu - G.So;
   } else {
     dq.rho = drho;
     dq.u = dun;
@@ -359,9 +327,12 @@ __device__ __forceinline__ void hlld_rev(const FaceState& sl, const FaceState& s
   dq.w = fma(dub, q.bz, fma(dru, q.w, dq.w));
   dq.by = fma(dub, q.v, dq.by);
   dq.bz = fma(dub, q.w, dq.bz);
-  dbn = fma(dub, q.u, fma(2.0 * bn, dbn2, dbn));
-  add_side(left, dsl, dsr, dq);
-  if (left) { dLb2 += deh; dLpt += dqpt; } else { dRb2 += deh; dRpt += dqpt; }
+  dbn = fma(dub, q.u, dbn);
+  G.left = left;
+  G.qa = dq;
+  G.qo = dqo;
+  G.pta = dqpt;
+  G.b2a = deh;
 }
 
 // Gradient of g = sum_v lf[v] F[v] + lap ap + lam am + lus u* of riemann<RS>(sl, sr, bn) in
@@ -370,32 +341,39 @@ template <int RS>
 __device__ __forceinline__ void riemann_vjp(const FaceState& sl, const FaceState& sr, double bn, double gam,
                                             double gm1inv, const double* lf, double lap, double lam, double lus,
                                             FaceState& dsl, FaceState& dsr, double& dbn) {
-  dsl = {0, 0, 0, 0, 0, 0, 0};
-  dsr = {0, 0, 0, 0, 0, 0, 0};
   dbn = 0.0;
+  const double bn2 = bn * bn;
+  double dbn2 = 0.0;
   // ---- forward (as in riemann) ----
   PhysFlux L, R;
-  phys_speed(sl, bn, gam, L);
-  phys_speed(sr, bn, gam, R);
-  double SL = 0.0, SR = 0.0, ap, am;
+  double SL = 0.0, SR = 0.0, ap, am, icmax = 0.0;
   bool llf_left = true, cmax_left = true, umax_left = true, umin_left = true, ap_pos = true, am_pos = true;
   if (RS == RS_LLF) {
+    phys_speed(sl, bn, gam, L);
+    phys_speed(sr, bn, gam, R);
     const double aL = vabs(sl.u) + sqrt_(L.cf2), aR = vabs(sr.u) + sqrt_(R.cf2);
     llf_left = dbits(aL) >= dbits(aR);
     ap = am = llf_left ? aL : aR;
   } else {
+    phys_speed_a(sl, bn2, gam, L);
+    phys_speed_a(sr, bn2, gam, R);
     bool fin;
     cmax_left = fast_left(sl, sr, L, R, fin);
-    const double cmax = fast_max(sl, sr, L, R);
+    // fast_max, and 1 / c from the same reciprocal root (0 where c is 0)
+    const double ah = halve(cmax_left ? L.A : R.A), rc = cmax_left ? sl.rho : sr.rho, x = ah * rc;
+    const double y = rsqrt_(x);
+    const bool z = is_zero(x);
+    const double cmax = !fin ? dfrom(0x7ff8000000000000LL) : (z ? 0.0 : vabs(ah) * y);
+    icmax = z ? 0.0 : rc * y;
     umax_left = okey(sl.u) >= okey(sr.u);
     umin_left = okey(sl.u) <= okey(sr.u);
     const double umax = umax_left ? sl.u : sr.u, umin = umin_left ? sl.u : sr.u;
     SR = umax + cmax;
     SL = umin - cmax;
     ap_pos = !(okey(0.0) >= okey(SR));  // vmax(0, SR) picks SR
-    am_pos = !(okey(0.0) >= okey(cmax - umin));
+    am_pos = !((unsigned long long)dbits(SL) <= 0x7ff0000000000000ULL);
     ap = ap_pos ? SR : 0.0;
-    am = am_pos ? cmax - umin : 0.0;
+    am = am_pos ? neg_if(dbits(SL) < 0, SL) : 0.0;
   }
   const double sum = ap + am;
   const bool zero = is_zero(sum);
@@ -403,26 +381,23 @@ __device__ __forceinline__ void riemann_vjp(const FaceState& sl, const FaceState
 
   // ---- reverse ----
   double dap = lap, dam = lam;
-  double dLb2 = 0.0, dLpt = 0.0, dRb2 = 0.0, dRpt = 0.0, dLcf = 0.0, dRcf = 0.0;
-  // u* = (ap uL + am uR) inv, or uL when ap + am = 0
-  if (zero) {
-    dsl.u += lus;
-  } else {
-    const double n = fma(ap, sl.u, am * sr.u);
-    const double dn = lus * inv;
-    const double dinv = lus * n;
-    dap += dn * sl.u;
-    dsl.u += dn * ap;
-    dam += dn * sr.u;
-    dsr.u += dn * am;
-    const double ds = -dinv * inv * inv;
-    dap += ds;
-    dam += ds;
-  }
+  double dLb2 = 0.0, dLpt = 0.0, dRb2 = 0.0, dRpt = 0.0;
   double dSL = 0.0, dSR = 0.0;
   if (RS == RS_HLLD) {
-    hlld_rev(sl, sr, bn, bn * bn, gm1inv, L, R, SL, SR, lf, dsl, dsr, dbn, dLb2, dLpt, dRb2, dRpt, dSL, dSR);
+    HlldAdj G;
+    hlld_rev(sl, sr, bn, bn2, gm1inv, L, R, SL, SR, lf, G, dbn, dbn2);
+    const bool l = G.left;
+    dsl = pick(l, G.qa, G.qo);
+    dsr = pick(l, G.qo, G.qa);
+    dLpt = l ? G.pta : G.pto;
+    dRpt = l ? G.pto : G.pta;
+    dLb2 = l ? G.b2a : 0.0;
+    dRb2 = l ? 0.0 : G.b2a;
+    dSL = l ? G.Sa : G.So;
+    dSR = l ? G.So : G.Sa;
   } else {
+    dsl = {0, 0, 0, 0, 0, 0, 0};
+    dsr = {0, 0, 0, 0, 0, 0, 0};
     phys_flux(sl, bn, gm1inv, L);
     phys_flux(sr, bn, gm1inv, R);
     double dUL[5], dFL[5], dUR[5], dFR[5];
@@ -451,35 +426,53 @@ __device__ __forceinline__ void riemann_vjp(const FaceState& sl, const FaceState
     phys_flux_rev(sl, bn, gm1inv, L, dUL, dFL, 0.0, dsl, dbn, dLb2, dLpt);
     phys_flux_rev(sr, bn, gm1inv, R, dUR, dFR, 0.0, dsr, dbn, dRb2, dRpt);
   }
+  // u* = (ap uL + am uR) inv, or uL when ap + am = 0
+  if (zero) {
+    dsl.u += lus;
+  } else {
+    const double dn = lus * inv;
+    const double ds = -(dn * fma(ap, sl.u, am * sr.u)) * inv;
+    dap += fma(dn, sl.u, ds);
+    dsl.u = fma(dn, ap, dsl.u);
+    dam += fma(dn, sr.u, ds);
+    dsr.u = fma(dn, am, dsr.u);
+  }
   // wave speeds
   if (RS == RS_LLF) {
     const double da = dap + dam;
-    if (llf_left) {
-      dsl.u += neg_if(dbits(sl.u) < 0, da);
-      dLcf += da;
-    } else {
-      dsr.u += neg_if(dbits(sr.u) < 0, da);
-      dRcf += da;
-    }
+    const double du = neg_if(dbits(llf_left ? sl.u : sr.u) < 0, da);
+    dsl.u += llf_left ? du : 0.0;
+    dsr.u += llf_left ? 0.0 : du;
+    // c = sqrt(cf2): derivative rsqrt / 2, taken as 0 at 0
+    const FaceState& q = llf_left ? sl : sr;
+    FaceState dq = {0, 0, 0, 0, 0, 0, 0};
+    const double cf2 = llf_left ? L.cf2 : R.cf2;
+    const double dcf2 = is_zero(cf2) ? 0.0 : 0.5 * rsqrt_(cf2) * da;
+    const double db2 = speed_rev(q, bn2, llf_left ? L.b2 : R.b2, llf_left ? L.A : R.A, gam, dcf2, dq, dbn2);
+    (llf_left ? dLb2 : dRb2) += db2;
+    (llf_left ? dsl : dsr).rho += dq.rho;
+    (llf_left ? dsl : dsr).p += dq.p;
   } else {
-    // ap = max(0, SR), am = max(0, cmax - umin), SR = umax + cmax, SL = umin - cmax
-    if (ap_pos) dSR += dap;
-    double dcmax = dSR - dSL, dumin = dSL;
-    const double dumax = dSR;
-    if (am_pos) {
-      dcmax += dam;
-      dumin -= dam;
-    }
-    if (cmax_left) dLcf += dcmax; else dRcf += dcmax;
-    if (umax_left) dsl.u += dumax; else dsr.u += dumax;
-    if (umin_left) dsl.u += dumin; else dsr.u += dumin;
+    // ap = max(0, SR), am = max(0, -SL), SR = umax + cmax, SL = umin - cmax
+    dSR += ap_pos ? dap : 0.0;
+    dSL -= am_pos ? dam : 0.0;
+    dsl.u += (umax_left ? dSR : 0.0) + (umin_left ? dSL : 0.0);
+    dsr.u += (umax_left ? 0.0 : dSR) + (umin_left ? 0.0 : dSL);
+    // the larger speed's side only: dcf2 = dc / (2 c)
+    const FaceState q = pick(cmax_left, sl, sr);
+    FaceState dq = {0, 0, 0, 0, 0, 0, 0};
+    const double db2 = speed_rev(q, bn2, cmax_left ? L.b2 : R.b2, cmax_left ? L.A : R.A, gam,
+                                 halve(icmax) * (dSR - dSL), dq, dbn2);
+    dLb2 += cmax_left ? db2 : 0.0;
+    dRb2 += cmax_left ? 0.0 : db2;
+    dsl.rho += cmax_left ? dq.rho : 0.0;
+    dsr.rho += cmax_left ? 0.0 : dq.rho;
+    dsl.p += cmax_left ? dq.p : 0.0;
+    dsr.p += cmax_left ? 0.0 : dq.p;
   }
-  // cf = sqrt(cf2) (the larger speed is the square root of the larger square): derivative
-  // rsqrt / 2, taken as 0 at 0
-  const double dLcf2 = is_zero(L.cf2) ? 0.0 : 0.5 * rsqrt_(L.cf2) * dLcf;
-  const double dRcf2 = is_zero(R.cf2) ? 0.0 : 0.5 * rsqrt_(R.cf2) * dRcf;
-  phys_speed_rev(sl, bn, gam, dLb2, dLpt, dLcf2, dsl, dbn);
-  phys_speed_rev(sr, bn, gam, dRb2, dRpt, dRcf2, dsr, dbn);
+  pt_rev(sl, dLb2, dLpt, dsl, dbn2);
+  pt_rev(sr, dRb2, dRpt, dsr, dbn2);
+  dbn = fma(2.0 * bn, dbn2, dbn);
 }
 
 }  // namespace mhd
