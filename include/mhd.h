@@ -128,7 +128,7 @@ mhd_status mhd_stats(mhd_ctx *ctx, long long *fofc_cells_stage1, long long *fofc
 enum {
   MHD_K_PRIM = 0,      /* cons -> prim */
   MHD_K_FACE = 1,      /* reconstruction + Riemann sweeps, 1 launch per stage (all directions) */
-  MHD_K_EDGE_BT = 2,   /* a-face quantities to edges along c, 1 launch per stage (B25a: + 6) */
+  MHD_K_EDGE_BT = 2,   /* a-face quantities to edges along c, 1 launch per stage (B25a: + 1) */
   MHD_K_EDGE_LR = 3,   /* c-face quantities to edges along a + LD04 + eta j, 1 per stage */
   MHD_K_UPDATE = 4,    /* flux divergence and CT update */
   MHD_K_FLAG = 5,      /* validity flags */

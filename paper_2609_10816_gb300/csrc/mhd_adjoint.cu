@@ -80,8 +80,8 @@ __device__ __forceinline__ void recon_jac(const double* q, double* JL, double* J
     const bool xa = ext_code(s0, s1, s2), xb = ext_code(s1, s2, s3);
     int pa, pb;  // 0: fourth-order value, 1: the lower cell's value, 2: the upper cell's
     double ra, sa, rb, sb;
-    ppm_ep_face(q[1], q[2], e0, e1, e2, xa && same_code(ka, kb), pa, ra, sa);
-    ppm_ep_face(q[2], q[3], e1, e2, e3, xb && same_code(kb, kc), pb, rb, sb);
+    ppm_ep_face<false>(q[1], q[2], e0, e1, e2, xa && same_code(ka, kb), pa, ra, sa);
+    ppm_ep_face<false>(q[2], q[3], e1, e2, e3, xb && same_code(kb, kc), pb, rb, sb);
     if (pa == 0) {
       JL[0] = -1.0 / 12.0; JL[1] = 7.0 / 12.0; JL[2] = 7.0 / 12.0; JL[3] = -1.0 / 12.0;
     } else {

@@ -129,9 +129,9 @@ void run_stage(mhd_ctx* c, const mhd::Dev& D, const Decoded& sc, PrimSource prim
   }
   { Timed t(c, MHD_K_FACE, D.work ? 1 : 3); mhd::launch_faces(D, sc.recon, sc.rs, c->seg, st); }
   {
-    // one launch per edge phase with work cursors (three without), B25a's six cell-to-face sweeps
+    // one launch per edge phase with work cursors (three without), B25a's cell-to-face sweeps one more
     const int n = D.work ? 1 : 3;
-    Timed t(c, MHD_K_EDGE_BT, sc.emf == mhd::EMF_B25A ? n + 6 : n);
+    Timed t(c, MHD_K_EDGE_BT, sc.emf == mhd::EMF_B25A ? n + 1 : n);
     mhd::launch_edges_bt(D, sc.recon, c->seg, st);
   }
   { Timed t(c, MHD_K_EDGE_LR, D.work ? 1 : 3); mhd::launch_edges_lr(D, sc.recon, c->seg, st); }

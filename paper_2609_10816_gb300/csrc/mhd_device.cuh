@@ -270,6 +270,7 @@ struct Line {
 // takes the value at m + LA and returns the left/right states of the interface between
 // points m-1 and m (left = upper value of point m-1, right = lower value of point m). Every
 // point's slope, interface value and limiter run exactly once per sweep.
+// FACE: the caller is a face sweep (PPM-EP's choice of pipe, ppm_ep_face).
 // For sweeps that keep their windows in shared memory: each() visits the NS doubles of the state,
 // and code holds NB more bits.
 // ------------------------------------------------------------------------------------------
@@ -280,7 +281,9 @@ template <> struct Rec<REC_PC> {
   double prev;
   int code;
   template <class F> __device__ __forceinline__ void each(F f) { f(0, prev); }
+  template <bool FACE>
   __device__ __forceinline__ void init(const double* q) { prev = q[0]; }
+  template <bool FACE>
   __device__ __forceinline__ void step(double qn, double& L, double& R) {
     L = prev;
     R = qn;
@@ -315,12 +318,14 @@ template <int R> struct RecPLM {
   __device__ __forceinline__ double hs(double a, double b) const {
     return R == REC_PLM_MC ? half_slope_mc(a, b) : half_slope_minmod(a, b);
   }
+  template <bool FACE>
   __device__ __forceinline__ void init(const double* q) {
     const double e0 = q[1] - q[0], e1 = q[2] - q[1];
     aRprev = q[1] + hs(e0, e1);
     qb = q[2];
     dl = e1;
   }
+  template <bool FACE>
   __device__ __forceinline__ void step(double qn, double& L, double& Rt) {
     const double dr = qn - qb;
     const double h = hs(dl, dr);
@@ -421,6 +426,13 @@ __host__ __device__ __forceinline__ unsigned long long fixed_to_bits(unsigned lo
 #endif
   return (((x + (1u << (sh - 1))) >> sh) + ((unsigned long long)(unsigned)(e - 8 + sh) << 52)) | sign;
 }
+// t / 12 to within 3, with 2^64 / 12 = 0x15555555_55555555
+__host__ __device__ __forceinline__ long long twelfth(long long t) {
+  const int th = (int)(t >> 32);
+  const unsigned tl = (unsigned)t;
+  return (long long)th * 0x15555555 + (long long)(((unsigned long long)tl * 0x15555555u) >> 32) +
+         (((long long)th * 0x55555555) >> 32);
+}
 // bit patterns of r and s from those of dl, d, dn, for the exponent field of d in [128, 2039] or
 // d = 0 (then both are 0)
 __host__ __device__ __forceinline__ void ppm_split_bits(unsigned long long bl, unsigned long long bd,
@@ -434,13 +446,7 @@ __host__ __device__ __forceinline__ void ppm_split_bits(unsigned long long bl, u
   if ((long long)(bn ^ bd) < 0) kn = 63;
   const unsigned long long fd = dmag_fixed(bd, 3);
   const unsigned long long d0 = fixed_slope2(dmag_fixed(bl, kl), fd), d1 = fixed_slope2(dmag_fixed(bn, kn), fd);
-  // t / 12 with 2^64 / 12 = 0x15555555_55555555
-  const long long t = (long long)(d0 - d1);
-  const int th = (int)(t >> 32);
-  const unsigned tl = (unsigned)t;
-  const long long q = (long long)th * 0x15555555 + (long long)(((unsigned long long)tl * 0x15555555u) >> 32) +
-                      (((long long)th * 0x55555555) >> 32);
-  const unsigned long long x = (fd >> 1) + (unsigned long long)q;
+  const unsigned long long x = (fd >> 1) + (unsigned long long)twelfth((long long)(d0 - d1));
   const unsigned long long sign = bd & 0x8000000000000000ULL;
   const bool zero = (bd << 1) == 0;
   r = zero ? 0 : fixed_to_bits(x, e, sign);
@@ -480,6 +486,7 @@ template <> struct Rec<REC_PPM> {
     f(5, f1);
     f(6, aRprev);
   }
+  template <bool FACE>
   __device__ __forceinline__ void init(const double* v) {  // v = q[m0-3 .. m0+1]
     const double e0 = v[1] - v[0], e1 = v[2] - v[1], e2 = v[3] - v[2], e3 = v[4] - v[3];
     double ra, sa, rb, sb;
@@ -496,6 +503,7 @@ template <> struct Rec<REC_PPM> {
     s2 = sb;
     f1 = fb;
   }
+  template <bool FACE>
   __device__ __forceinline__ void step(double qn, double& L, double& R) {
     const double dn = qn - q2;
     double r, s;
@@ -545,13 +553,70 @@ __device__ __forceinline__ int median3_pick(T a, T b, T c) {
   return klo >= km ? lo : m;
 }
 // The fourth-order value (7 (qa + qb) - (qc + qd)) / 12 lies r = d/2 + (dl - dn)/12 above qa, with
-// d = qb - qa and the differences dl before qa and dn after qb.
-// r and s = qb - f of the interface between qa and qb (f = qa + r); keep: it lies at a smooth
+// d = qb - qa and the differences dl before qa and dn after qb, and s = d - r below qb. Formed on the
+// integer pipe like PPM's (ppm_split_bits): the three differences are shifted to the largest one's
+// exponent (its significand times 2^7), so r and s are good to 2^-58 of it before their one rounding
+// (FP64 instructions round three times at 2^-53 of d and dl - dn), and two FP64 instructions fewer
+// are issued per value than with the sum formed in FP64.
+__host__ __device__ __forceinline__ long long dsigned_fixed(unsigned long long b, int right) {
+  const unsigned long long m = (((b & 0x000fffffffffffffULL) | 0x0010000000000000ULL) << 7) >> (right > 63 ? 63 : right);
+  return (long long)b < 0 ? -(long long)m : (long long)m;
+}
+// the double nearest to x 2^(e - 1082), for |x| < 2^62 and e >= 128
+__host__ __device__ __forceinline__ unsigned long long signed_fixed_to_bits(long long x, int e) {
+  const unsigned long long m = (unsigned long long)(x < 0 ? -x : x);
+  if (m == 0) return 0;
+#ifdef __CUDA_ARCH__
+  const int sh = 11 - __clzll((long long)m);  // the leading bit to bit 52
+#else
+  const int sh = 11 - __builtin_clzll(m);
+#endif
+  const unsigned long long q = sh > 0 ? (m + (1ULL << (sh - 1))) >> sh : m << -sh;
+  return (q + ((unsigned long long)(unsigned)(e - 8 + sh) << 52)) | ((unsigned long long)x & 0x8000000000000000ULL);
+}
+// bit patterns of r and s from those of dl, d, dn, for the largest exponent field e of the three in
+// [128, 2039]
+__host__ __device__ __forceinline__ void ppm_ep_split_bits(unsigned long long bl, unsigned long long bd,
+                                                           unsigned long long bn, int e, int el, int ed, int en,
+                                                           unsigned long long& r, unsigned long long& s) {
+  const long long fl = dsigned_fixed(bl, e - el), fd = dsigned_fixed(bd, e - ed), fn = dsigned_fixed(bn, e - en);
+  const long long x = (fd >> 1) + twelfth(fl - fn);
+  r = signed_fixed_to_bits(x, e);
+  s = signed_fixed_to_bits(fd - x, e);
+}
+static __device__ __noinline__ double ppm_ep_offset_any(double dl, double d, double dn) {
+  return fma(dl - dn, 1.0 / 12.0, halve(d));
+}
+__device__ __forceinline__ void ppm_ep_split(double dl, double d, double dn, double& r, double& s) {
+  const unsigned long long bl = (unsigned long long)dbits(dl), bd = (unsigned long long)dbits(d),
+                           bn = (unsigned long long)dbits(dn);
+  const int el = (int)(bl >> 52) & 0x7ff, ed = (int)(bd >> 52) & 0x7ff, en = (int)(bn >> 52) & 0x7ff;
+  const int e = max(ed, max(el, en));
+  if ((unsigned)e - 128u > 1911u) {
+    const bool zero = ((bl | bd | bn) << 1) == 0;
+    r = zero ? 0.0 : ppm_ep_offset_any(dl, d, dn);
+    s = zero ? 0.0 : __dsub_rn(d, r);
+    return;
+  }
+  unsigned long long br, bs;
+  ppm_ep_split_bits(bl, bd, bn, e, el, ed, en, br, bs);
+  r = dfrom((long long)br);
+  s = dfrom((long long)bs);
+}
+// r and s of the interface between qa and qb (f = qa + r); keep: it lies at a smooth
 // extremum (no bound), else f is bounded by the two cells. pick: 0 the fourth-order value, 1 qa, 2 qb.
+// FIXED: r and s on the integer pipe. The face sweeps take that form (128^3 Alfven wave: 3.97 ms a step
+// against 4.29), the edge sweeps the FP64 one: they do little else, and the integer pipe would bound
+// them (bottom/top 0.53 ms against 0.38, with B25a's sweeps at 96^3 0.69 against 0.58).
+template <bool FIXED>
 __device__ __forceinline__ double ppm_ep_face(double qa, double qb, double dl, double d, double dn, bool keep,
                                               int& pick, double& r, double& s) {
-  r = fma(dl - dn, 1.0 / 12.0, halve(d));
-  s = d - r;
+  if (FIXED) {
+    ppm_ep_split(dl, d, dn, r, s);
+  } else {
+    r = fma(dl - dn, 1.0 / 12.0, halve(d));
+    s = __dsub_rn(d, r);
+  }
   const double f = qa + r;
   pick = 0;
   if (!keep) {
@@ -590,6 +655,7 @@ template <> struct Rec<REC_PPM_EP> {
     f(5, f1);
     f(6, aRprev);
   }
+  template <bool FACE>
   __device__ __forceinline__ void init(const double* v) {  // v = q[m0-3 .. m0+1]
     const double e0 = v[1] - v[0], e1 = v[2] - v[1], e2 = v[3] - v[2], e3 = v[4] - v[3];
     const int s0 = sgn_code(e0), s1 = sgn_code(e1), sb = sgn_code(e2), s3 = sgn_code(e3);
@@ -598,8 +664,8 @@ template <> struct Rec<REC_PPM_EP> {
     const bool xa = ext_code(s0, s1, sb), xb = ext_code(s1, sb, s3);
     int p;
     double ra, sa, rb;
-    const double fa = ppm_ep_face(v[1], v[2], e0, e1, e2, xa && same_code(ka, kb), p, ra, sa);   // m0 - 3/2
-    const double fb = ppm_ep_face(v[2], v[3], e1, e2, e3, xb && same_code(kb, kc), p, rb, s2);  // m0 - 1/2
+    const double fa = ppm_ep_face<FACE>(v[1], v[2], e0, e1, e2, xa && same_code(ka, kb), p, ra, sa);   // m0 - 3/2
+    const double fb = ppm_ep_face<FACE>(v[2], v[3], e1, e2, e3, xb && same_code(kb, kc), p, rb, s2);  // m0 - 1/2
     double aL = fa, aR = fb;
     if (!((xa || xb) && same_code(ka, kb) && same_code(kb, kc))) ppm_mono(v[2], rb, sa, aL, aR);
     aRprev = aR;
@@ -610,6 +676,7 @@ template <> struct Rec<REC_PPM_EP> {
     f1 = fb;
     code = kb | ((int)xb << 2);
   }
+  template <bool FACE>
   __device__ __forceinline__ void step(double qn, double& L, double& R) {
     const double dn = qn - q2;  // q[m+2] - q[m+1]
     const int c0 = code & 3, c1 = cmp_code(dq, dl), cn = cmp_code(dn, dq);  // points m-1, m, m+1
@@ -617,7 +684,7 @@ template <> struct Rec<REC_PPM_EP> {
     const bool x2 = ext_code(sgn_code(dl), sgn_code(dq), sgn_code(dn));
     int p;
     double r, s;
-    const double f2 = ppm_ep_face(q1, q2, dl, dq, dn, x2 && same_code(c1, cn), p, r, s);  // m + 1/2
+    const double f2 = ppm_ep_face<FACE>(q1, q2, dl, dq, dn, x2 && same_code(c1, cn), p, r, s);  // m + 1/2
     double aL = f1, aR = f2;
     if (!((x1 || x2) && same_code(c0, c1) && same_code(c1, cn))) ppm_mono(q1, r, s2, aL, aR);
     L = aRprev;
@@ -709,7 +776,7 @@ template <> struct LaneRec<REC_PPM_EP> {
     const bool x2 = ext_code(sgn_code(dl), sgn_code(dq), sgn_code(dn));
     int p;
     double r, s;
-    const double f2 = ppm_ep_face(q[0], q[1], dl, dq, dn, x2 && same_code(c1, cn), p, r, s);
+    const double f2 = ppm_ep_face<true>(q[0], q[1], dl, dq, dn, x2 && same_code(c1, cn), p, r, s);
     const double s2 = w.up1(s, prev[1]);
     double aL = w.up1(f2, prev[2]), aR = f2;
     const int mine = c1 | ((int)x2 << 2), before = w.up1(mine, code);
@@ -984,11 +1051,11 @@ __device__ __forceinline__ void hlld(const FaceStateT<T>& sl, const FaceStateT<T
   F[4] = fma(e + pt, un, -(ub * bn));
 }
 
-// Full face solve: flux of {rho, m_n, m_t1, m_t2, e}, alpha+/-, and the Q26 face velocity.
+// Full face solve: flux of {rho, m_n, m_t1, m_t2, e}, alpha+/-, and (with_us) the Q26 face velocity.
 template <int RS, class T>
 __device__ __forceinline__ void riemann(const FaceStateT<T>& sl, const FaceStateT<T>& sr, T bn,
                                         double gam, double gm1inv, T* F, T& ap,
-                                        T& am, T& ustar) {
+                                        T& am, T& ustar, bool with_us = true) {
   PhysFluxT<T> L, R;
   const T bn2 = bn * bn;
   T SL = 0.0, SR = 0.0;
@@ -1010,12 +1077,14 @@ __device__ __forceinline__ void riemann(const FaceStateT<T>& sl, const FaceState
     // max(0, -SL), a speed that is not a number kept: -SL is cmax - umin, without forming it
     am = (unsigned long long)dbits(val(SL)) <= 0x7ff0000000000000ULL ? T(0.0) : neg_if(dbits(val(SL)) < 0, SL);
   }
+  if (RS == RS_HLLD) {
+    hlld(sl, sr, bn, bn2, gm1inv, L, R, SL, SR, F);  // (reads L, R's pt and b2 only)
+    if (!with_us) return;
+  }
   const T sum = ap + am;
   const bool zero = is_zero(sum);
   const T inv = zero ? 0.0 : rcp(sum);
-  if (RS == RS_HLLD) {
-    hlld(sl, sr, bn, bn2, gm1inv, L, R, SL, SR, F);  // (reads L, R's pt and b2 only)
-  } else {
+  if (RS != RS_HLLD) {
     phys_flux(sl, bn, gm1inv, L);
     phys_flux(sr, bn, gm1inv, R);
     two_state(L, R, ap, am, inv, zero, F);

@@ -15,13 +15,32 @@ __global__ void __launch_bounds__(128) k_edge_bt(Dev D, int e, int seg) {
   edge_bt_seg<RC, EMF>(D, e, ln, m0, m1);
 }
 
+// B25a's six sweeps of the cell EMFs to faces (for every direction the EMF reconstructed along it as
+// the "a" direction and the one as the "c" direction) as one persistent launch: apart, each left most
+// of the GPU idle (96^3, bottom/top sweeps and these: 1.02 ms a step, so 0.58).
 template <int RC>
-__global__ void __launch_bounds__(128) k_b25_cell_to_face(Dev D, int e, int to_a, int seg) {
-  Line ln;
-  int m0, m1;
-  const int dir = to_a ? (e + 1) % 3 : (e + 2) % 3;
-  if (!sweep_line(D, dir, seg, ln, m0, m1, dir == 0)) return;
-  b25_seg<RC>(D, e, to_a, ln, m0, m1);
+__global__ void __launch_bounds__(128) k_b25_cell_to_face(Dev D, int s0, int s1, int s2) {
+  const int sg[3] = {s0, s1, s2};
+  long long tot[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) tot[d] = sweep_threads(D, d, sg[d]);
+  for_each_segment(work_cursor(D, CUR_B25A), 2 * (tot[0] + tot[1] + tot[2]), [&](long long t) {
+    int dir = 0;
+    if (t >= 2 * tot[0]) {
+      t -= 2 * tot[0];
+      dir = 1;
+      if (t >= 2 * tot[1]) {
+        t -= 2 * tot[1];
+        dir = 2;
+      }
+    }
+    const int to_a = t < tot[dir];
+    if (!to_a) t -= tot[dir];
+    Line ln;
+    int m0, m1;
+    if (sweep_line_at(D, dir, sg[dir], t, ln, m0, m1, dir == 0, dir != 0))
+      b25_seg<RC>(D, to_a ? (dir + 2) % 3 : (dir + 1) % 3, to_a, ln, m0, m1);
+  });
 }
 
 template <int RC, int EMF>
@@ -108,13 +127,15 @@ static void launch_lr_t(const Dev& d, int seg, cudaStream_t st) {
 template <int RC>
 static void launch_b25_t(const Dev& d, int seg, cudaStream_t st) {
   const int bs = 128;
-  for (int e = 0; e < 3; ++e)
-    for (int to_a = 0; to_a < 2; ++to_a) {
-      const int dir = to_a ? (e + 1) % 3 : (e + 2) % 3;
-      const int sg = edge_sweep_seg(d, dir, seg);
-      const long long th = sweep_threads(d, dir, sg);
-      k_b25_cell_to_face<RC><<<(unsigned)((th + bs - 1) / bs), bs, 0, st>>>(d, e, to_a, sg);
-    }
+  const long long res = resident_blocks((const void*)k_b25_cell_to_face<RC>, bs);
+  int sg[3];
+  long long tot = 0;
+  for (int dir = 0; dir < 3; ++dir) {
+    sg[dir] = edge_sweep_seg(d, dir, seg);
+    if (dir != 0) sg[dir] = fill_seg(d, dir, sg[dir], res * bs);
+    tot += 2 * sweep_threads(d, dir, sg[dir]);
+  }
+  k_b25_cell_to_face<RC><<<(unsigned)std::min((tot + bs - 1) / bs, res), bs, 0, st>>>(d, sg[0], sg[1], sg[2]);
 }
 
 template <int RC>

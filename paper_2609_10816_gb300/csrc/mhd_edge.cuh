@@ -65,7 +65,7 @@ __device__ __forceinline__ void edge_bt_seg(const Dev& D, int e, const Line& ln,
     double w[LB + LA];
 #pragma unroll
     for (int t = 0; t < LB + LA; ++t) w[t] = q[v][ln.at(m0 - LB + t)];
-    r[v].init(w);
+    r[v].template init<false>(w);
   }
   // the next point's values are loaded one iteration ahead (this sweep does little arithmetic per
   // point, so the loads' latency would otherwise stall it)
@@ -85,7 +85,7 @@ __device__ __forceinline__ void edge_bt_seg(const Dev& D, int e, const Line& ln,
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       double B, T;
-      r[v].step(cur[v], B, T);
+      r[v].template step<false>(cur[v], B, T);
       out[2 * v][X] = B;
       out[2 * v + 1][X] = T;
     }
@@ -110,11 +110,11 @@ __device__ __forceinline__ void b25_seg(const Dev& D, int e, int to_a, const Lin
   double w[LB + LA];
 #pragma unroll
   for (int t = 0; t < LB + LA; ++t) w[t] = eps(ln.at(m0 - LB + t));
-  r.init(w);
+  r.template init<false>(w);
   for (int m = m0; m < m1; ++m) {
     const long long X = ln.at(m);
     double lo, hi;
-    r.step(eps(ln.at(m + LA)), lo, hi);
+    r.template step<false>(eps(ln.at(m + LA)), lo, hi);
     out[X] = lo;
     out[N + X] = hi;
   }
@@ -184,7 +184,7 @@ __device__ __forceinline__ void edge_lr_seg(const Dev& D, int e, const Line& ln,
     double w[LB + LA];
 #pragma unroll
     for (int t = 0; t < LB + LA; ++t) w[t] = q[v][ln.at(m0 - LB + t)];
-    r[v].init(w);
+    r[v].template init<false>(w);
   }
   const double* part = D.Epart + 4LL * e * N;
   const double* xp = D.Xpart + 8LL * e * N;
@@ -202,7 +202,7 @@ __device__ __forceinline__ void edge_lr_seg(const Dev& D, int e, const Line& ln,
     const long long Xn = ln.at(m + LA);
     double lo[NV], hi[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) r[v].step(q[v][Xn], lo[v], hi[v]);
+    for (int v = 0; v < NV; ++v) r[v].template step<false>(q[v][Xn], lo[v], hi[v]);
     const double bcL = lo[0], bcR = hi[0];
     const double baB = part[0 * N + X], baT = part[1 * N + X];
     // Eq. (alpha-edge): alpha_a from the two a-faces (c-neighbours), alpha_c from the c-faces

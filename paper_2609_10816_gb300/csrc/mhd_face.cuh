@@ -80,11 +80,11 @@ __device__ __forceinline__ void face_solve(const Dev& D, int dir, long long X, c
   }
   const FaceState sl = {Lv[0], Lv[1], Lv[2], Lv[3], Lv[4], Lv[5], Lv[6]};
   const FaceState sr = {Rv[0], Rv[1], Rv[2], Rv[3], Rv[4], Rv[5], Rv[6]};
-  double f[5], ap, am, us;
-  riemann<RS>(sl, sr, D.Bin[dir][X], D.gam, D.gm1inv, f, ap, am, us);
+  double f[5], ap, am, us = 0.0;
+  riemann<RS>(sl, sr, D.Bin[dir][X], D.gam, D.gm1inv, f, ap, am, us, D.emf == EMF_Q26);
   D.Ap[dir * N + X] = ap;
   D.Am[dir * N + X] = am;
-  D.Us[dir * N + X] = us;
+  if (D.emf == EMF_Q26) D.Us[dir * N + X] = us;
   if (D.resistive) f[4] += joule_flux(D, dir, X);
   if (D.combine) {
 #pragma unroll
@@ -126,7 +126,7 @@ __device__ __forceinline__ void face_piece(const Dev& D, int dir, bool by_lanes,
       for (int t = 0; t < LB + LA; ++t) p[t] = q[ln.at(m0 - LB + t)];
       Rec<RC> r;
       r.code = 0;
-      r.init(p);
+      r.template init<true>(p);
       r.each([&](int k, double& x) { win[k * ST + v * kFaceThreads] = x; });
       if (NB > 0) codes |= (unsigned)r.code << (NB * v);
     }
@@ -185,7 +185,7 @@ __device__ __forceinline__ void face_piece(const Dev& D, int dir, bool by_lanes,
         const double q = qn;
         if (v < 6) qn = P[((rows >> (4 * v + 4)) & 7) * N];
         double lv, rv;
-        r.step(q, lv, rv);
+        r.template step<true>(q, lv, rv);
         r.each([&](int k, double& x) { slot[k * ST] = x; });
         slot[NS * ST] = lv;
         slot[(NS + 1) * ST] = rv;

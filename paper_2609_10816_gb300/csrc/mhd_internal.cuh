@@ -79,7 +79,7 @@ inline void set_eta(Dev& D, double eta) {
 // Counters and cursors of a context: 8 counters, then 8 cursors, cleared by one memset per step.
 constexpr int kCounters = 8;
 constexpr int kWorkSlots = 8;
-enum { CUR_FACE = 0, CUR_EDGE_BT = 1, CUR_EDGE_LR = 2 };
+enum { CUR_FACE = 0, CUR_EDGE_BT = 1, CUR_EDGE_LR = 2, CUR_B25A = 3 };
 // the cursor of one sweep launch (each has its own per stage, so that they need no clearing between)
 __host__ __device__ inline unsigned long long* work_cursor(const Dev& D, int sweep) {
   return D.work + 4 * D.stage + sweep;
