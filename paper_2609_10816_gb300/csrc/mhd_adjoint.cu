@@ -319,14 +319,12 @@ __global__ void __launch_bounds__(128) k_adj_edges(AdjDev A) {
   const long long X = aid();
   const long long N = D.N;
   double etaacc = 0.0;
-  for (int e = 0; e < 3 && X < N; ++e) {  // no early return: the whole warp sums d/d(eta) below
-    const int a = (e + 1) % 3, c = (e + 2) % 3;
-    constexpr int NE = EMF == EMF_FS18 ? 20 : (EMF == EMF_B25A ? 12 : 8);  // adjoint slots per edge
-    const double lam = A.lE[e * N + X];
-    if (lam == 0.0) {
-      for (int k = 0; k < NE; ++k) A.lEdge[(NE * e + k) * N + X] = 0.0;
-      continue;
-    }
+  const int e = blockIdx.y, a = (e + 1) % 3, c = (e + 2) % 3;
+  constexpr int NE = EMF == EMF_FS18 ? 20 : (EMF == EMF_B25A ? 12 : 8);  // adjoint slots per edge
+  const double lam = X < N ? A.lE[e * N + X] : 0.0;
+  if (X < N && lam == 0.0)
+    for (int k = 0; k < NE; ++k) A.lEdge[(NE * e + k) * N + X] = 0.0;
+  if (lam != 0.0) {  // no early return: the whole warp sums d/d(eta) below
     const long long Xc = shift(D, X, c, -1), Xa = shift(D, X, a, -1);
     // the reconstructed edge values as the forward edge sweeps formed them. Q26: b_a, u_a* bottom
     // and top (Epart), b_c, u_c* left and right (EdgeC). FS18: b_a bottom and top (Epart), b_c
@@ -415,6 +413,11 @@ __global__ void __launch_bounds__(128) k_adj_edges(AdjDev A) {
 __device__ constexpr int kFs18RowBt[4] = {1, 8, 2, 9};
 __device__ constexpr int kFs18RowLr[4] = {3, 10, 1, 8};
 
+// (one face direction and one of its sources per blockIdx.y: small boxes have too few cells for a
+// thread to take them all in turn)
+template <int EMF> struct EdgeRecSources {
+  static constexpr int NB = EMF == EMF_Q26 ? 2 : (EMF == EMF_FS18 ? 5 : 3);  // per reconstruction direction
+};
 template <int RC, int EMF>
 __global__ void __launch_bounds__(128) k_adj_edge_rec(AdjDev A) {
   const Dev& D = A.D;
@@ -422,39 +425,40 @@ __global__ void __launch_bounds__(128) k_adj_edge_rec(AdjDev A) {
   if (X >= D.N) return;
   const long long N = D.N;
   constexpr int NE = EMF == EMF_FS18 ? 20 : (EMF == EMF_B25A ? 12 : 8);
-  for (int d = 0; d < 3; ++d) {
-    const int t1 = (d + 1) % 3, e1 = (d + 2) % 3;  // d is "a" of e1, reconstructed along c(e1) = t1
-    const int t2 = (d + 2) % 3, e2 = (d + 1) % 3;  // d is "c" of e2, reconstructed along a(e2) = t2
-    const double* L1 = A.lEdge + (long long)NE * e1 * N;
-    const double* L2 = A.lEdge + (long long)NE * e2 * N;
-    const long long X1 = shift(D, X, t1, 1), X2 = shift(D, X, t2, 1);
-    // point X's lower value is the top (right) value at edge X, its upper value the bottom (left)
-    // value at edge X + t
-    if (EMF == EMF_B25A) {  // b_d, and the e-EMF face values EfL (d = a of e1) and EfB (d = c of e2)
-      rec_scatter<RC>(D, D.Bin[d], X, t1, L1[1 * N + X], L1[0 * N + X1], A.lB + d * N);
-      rec_scatter<RC>(D, D.Bin[d], X, t2, L2[3 * N + X], L2[2 * N + X2], A.lB + d * N);
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const long long r1 = (2LL * e1 + k) * N, r2 = (2LL * e2 + k) * N;
-        rec_scatter<RC>(D, D.EfL + r1, X, t1, L1[(5 + 2 * k) * N + X], L1[(4 + 2 * k) * N + X1], A.lEf + r1);
-        rec_scatter<RC>(D, D.EfB + r2, X, t2, L2[(9 + 2 * k) * N + X], L2[(8 + 2 * k) * N + X2], A.lEf + 6 * N + r2);
-      }
-    } else if (EMF == EMF_FS18) {
-      rec_scatter<RC>(D, D.Bin[d], X, t1, L1[1 * N + X], L1[0 * N + X1], A.lB + d * N);
-      rec_scatter<RC>(D, D.Bin[d], X, t2, L2[3 * N + X], L2[2 * N + X2], A.lB + d * N);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const long long rb = (14LL * d + kFs18RowBt[k]) * N, rl = (14LL * d + kFs18RowLr[k]) * N;
-        rec_scatter<RC>(D, D.LR + rb, X, t1, L1[(5 + 2 * k) * N + X], L1[(4 + 2 * k) * N + X1], A.lLR + rb);
-        rec_scatter<RC>(D, D.LR + rl, X, t2, L2[(13 + 2 * k) * N + X], L2[(12 + 2 * k) * N + X2], A.lLR + rl);
-      }
-    } else {
-      rec_scatter<RC>(D, D.Bin[d], X, t1, L1[1 * N + X], L1[0 * N + X1], A.lB + d * N);
-      rec_scatter<RC>(D, D.Bin[d], X, t2, L2[5 * N + X], L2[4 * N + X2], A.lB + d * N);
-      rec_scatter<RC>(D, D.Us + d * N, X, t1, L1[3 * N + X], L1[2 * N + X1], A.lUs + d * N);
-      rec_scatter<RC>(D, D.Us + d * N, X, t2, L2[7 * N + X], L2[6 * N + X2], A.lUs + d * N);
-    }
+  constexpr int NB = EdgeRecSources<EMF>::NB;
+  const int d = blockIdx.y / (2 * NB), r = blockIdx.y % (2 * NB);
+  const bool bt = r < NB;
+  const int k = bt ? r : r - NB;  // 0: b_d, then the scheme's sources
+  // d is "a" of the e-edges with e = d + 2, reconstructed along t = c(e) = d + 1, or "c" of those with
+  // e = d + 1, reconstructed along t = a(e) = d + 2
+  const int t = (d + (bt ? 1 : 2)) % 3, e = (d + (bt ? 2 : 1)) % 3;
+  const double* L = A.lEdge + (long long)NE * e * N;
+  const long long Xt = shift(D, X, t, 1);
+  // point X's lower value is the top (right) value at edge X, its upper value the bottom (left)
+  // value at edge X + t: slots hi and hi - 1
+  int hi;
+  const double* q;
+  double* out;
+  if (k == 0) {
+    hi = EMF == EMF_Q26 ? (bt ? 1 : 5) : (bt ? 1 : 3);
+    q = D.Bin[d];
+    out = A.lB + d * N;
+  } else if (EMF == EMF_Q26) {
+    hi = bt ? 3 : 7;
+    q = D.Us + d * N;
+    out = A.lUs + d * N;
+  } else if (EMF == EMF_B25A) {  // the e-EMF face values EfL (d = a of e) or EfB (d = c of e)
+    const long long row = (2LL * e + k - 1) * N;
+    hi = (bt ? 5 : 9) + 2 * (k - 1);
+    q = (bt ? D.EfL : D.EfB) + row;
+    out = A.lEf + (bt ? 0 : 6 * N) + row;
+  } else {  // FS18's velocity states
+    const long long row = (14LL * d + (bt ? kFs18RowBt[k - 1] : kFs18RowLr[k - 1])) * N;
+    hi = (bt ? 5 : 13) + 2 * (k - 1);
+    q = D.LR + row;
+    out = A.lLR + row;
   }
+  rec_scatter<RC>(D, q, X, t, L[hi * N + X], L[(hi - 1) * N + Xt], out);
 }
 
 // ---- reconstructions as reverse sweeps (PPM) ------------------------------------------------
@@ -839,21 +843,20 @@ __global__ void __launch_bounds__(128) k_adj_joule(AdjDev A) {
   warp_add(deta, A.lEta);
 }
 // ---- face reconstructions: adjoint of the primitives --------------------------------------
+// (one direction and variable per blockIdx.y)
 template <int RC>
 __global__ void __launch_bounds__(128) k_adj_face_rec(AdjDev A) {
   const Dev& D = A.D;
   const long long X = aid();
   if (X >= D.N) return;
   const long long N = D.N;
-  for (int dir = 0; dir < 3; ++dir) {
-    const int a = (dir + 1) % 3, c = (dir + 2) % 3;
-    const int slot[7] = {0, 1 + dir, 1 + a, 1 + c, 4, 5 + a, 5 + c};
-    const double* lLR = A.lLR + 14LL * dir * N;
-    const long long Xn = shift(D, X, dir, 1);
-    // point X's lower value = right state of face X, upper value = left state of face X + dir
-    for (int v = 0; v < 7; ++v)
-      rec_scatter<RC>(D, D.P + slot[v] * N, X, dir, lLR[(7 + v) * N + X], lLR[v * N + Xn], A.lP + slot[v] * N);
-  }
+  const int dir = blockIdx.y / 7, v = blockIdx.y % 7;
+  const int a = (dir + 1) % 3, c = (dir + 2) % 3;
+  const int slot = v == 0 ? 0 : v == 1 ? 1 + dir : v == 2 ? 1 + a : v == 3 ? 1 + c : v == 4 ? 4 : v == 5 ? 5 + a : 5 + c;
+  const double* lLR = A.lLR + 14LL * dir * N;
+  const long long Xn = shift(D, X, dir, 1);
+  // point X's lower value = right state of face X, upper value = left state of face X + dir
+  rec_scatter<RC>(D, D.P + slot * N, X, dir, lLR[(7 + v) * N + X], lLR[v * N + Xn], A.lP + slot * N);
 }
 
 // ---- primitives: adjoint of cons -> prim ------------------------------------------------
@@ -1224,9 +1227,9 @@ static void adj_edges_t(const AdjDev& A, cudaStream_t st) {
     cudaMemsetAsync(A.leps, 0, 3 * A.D.N * sizeof(double), st);
     k_adj_eps_prep<<<nb256, 256, 0, st>>>(A);
   }
-  k_adj_edges<RC, EMF><<<nb, 128, 0, st>>>(A);
+  k_adj_edges<RC, EMF><<<dim3(nb, 3), 128, 0, st>>>(A);
   if (RC == REC_PPM) rec_sweeps<0, EMF>(A, st);
-  else k_adj_edge_rec<RC, EMF><<<nb, 128, 0, st>>>(A);
+  else k_adj_edge_rec<RC, EMF><<<dim3(nb, 6 * EdgeRecSources<EMF>::NB), 128, 0, st>>>(A);
   if (EMF == EMF_B25A) {  // the face EMF values back to the cell EMF, then to the primitives
     if (RC == REC_PPM) rec_sweeps<2>(A, st);
     else k_adj_eps_rec<RC><<<nb, 128, 0, st>>>(A);
@@ -1249,7 +1252,7 @@ static void adj_flux_r(const AdjDev& A, int rs, cudaStream_t st) {
   else k_adj_faces<RC, RS_LLF><<<nb3, 128, 0, st>>>(A);
   if (A.D.resistive) k_adj_joule<<<nb3, 128, 0, st>>>(A);
   if (RC == REC_PPM) rec_sweeps<1>(A, st);
-  else k_adj_face_rec<RC><<<nb, 128, 0, st>>>(A);
+  else k_adj_face_rec<RC><<<dim3(nb, 21), 128, 0, st>>>(A);
   k_adj_prim<<<nb, 128, 0, st>>>(A);
 }
 
