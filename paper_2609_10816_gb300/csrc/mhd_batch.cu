@@ -38,17 +38,14 @@ __global__ void __launch_bounds__(256) k_batch_maxspeed(BatchDev B) {
   double s = 0.0;
   for (long long base = t0 - lane; base < ncell; base += nth) {  // uniform over the warp
     const long long i = base + lane;
+    const double m = warp_max_enter(s, B.counters + 2);
+    s = m;
     if (i < ncell) {
       k = advance_pos(B.cell_pref, k, i);
       const Dev& D = B.patches[B.order[k]];
-      s = cfl_speed_max(D, D.U0, D.B0, i - B.cell_pref[k], s, D.P);  // and stage 1's primitives
+      s = cfl_speed_max(D, D.U0, D.B0, i - B.cell_pref[k], m, D.P);  // and stage 1's primitives
     }
-    unsigned long long b = (unsigned long long)dbits(s);
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long t = __shfl_xor_sync(0xffffffffu, b, o);
-      b = t > b ? t : b;
-    }
-    s = __longlong_as_double((long long)b);
+    s = warp_max_leave(s, m, B.counters + 2);
   }
   // block max then one atomic
   unsigned long long bits = (unsigned long long)dbits(s);

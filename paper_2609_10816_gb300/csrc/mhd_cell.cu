@@ -92,25 +92,24 @@ __device__ __forceinline__ void block_max_atomic(double v, unsigned long long* o
   __syncthreads();  // sm[] may be reused by a following call
 }
 
-// max over a thread's cells of the CFL signal speed (cfl_speed_max): a grid-stride loop whose warps
-// share their running maximum after every pass, so that most cells are settled by the bound check
-__device__ __forceinline__ double cell_speed_max(const Dev& D, const double* U, const Ptr3& Bp, double* Pout) {
+// max over a thread's cells of the CFL signal speed (cfl_speed_max), and over the cells that the grid
+// has judged so far: a grid-stride loop whose warps share their running maximum through *out, so that
+// most cells are settled by the bound checks
+__device__ __forceinline__ double cell_speed_max(const Dev& D, const double* U, const Ptr3& Bp, double* Pout,
+                                                 unsigned long long* out) {
   const long long nth = (long long)gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31;
   double s = 0.0;
   for (long long base = cell_id() - lane; base < D.N; base += nth) {  // uniform over the warp
-    if (base + lane < D.N) s = cfl_speed_max(D, U, Bp.p, base + lane, s, Pout);
-    unsigned long long b = (unsigned long long)dbits(s);
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long t = __shfl_xor_sync(0xffffffffu, b, o);
-      b = t > b ? t : b;
-    }
-    s = __longlong_as_double((long long)b);
+    const double m = warp_max_enter(s, out);
+    s = m;
+    if (base + lane < D.N) s = cfl_speed_max(D, U, Bp.p, base + lane, m, Pout);
+    s = warp_max_leave(s, m, out);
   }
   return s;
 }
 __global__ void __launch_bounds__(256) k_maxspeed(Dev D, const double* U, Ptr3 Bp, unsigned long long* out) {
-  block_max_atomic(cell_speed_max(D, U, Bp, nullptr), out);
+  block_max_atomic(cell_speed_max(D, U, Bp, nullptr, out), out);
 }
 
 // The same reduction, with S^n's primitives, and dt by the last block to finish (the operations of
@@ -129,7 +128,7 @@ __device__ __forceinline__ void set_dt(const Dev& D, const DtArgs& a, double sma
 }
 __global__ void __launch_bounds__(256) k_maxspeed_dt(Dev D, const double* U, Ptr3 Bp, unsigned long long* smax,
                                                      DtArgs a) {
-  block_max_atomic(cell_speed_max(D, U, Bp, D.P), smax);
+  block_max_atomic(cell_speed_max(D, U, Bp, D.P, smax), smax);
   if (threadIdx.x == 0) {
     __threadfence();
     if (atomicAdd(a.done, 1ull) == gridDim.x - 1) set_dt(D, a, dfrom((long long)atomicMax(smax, 0ull)));

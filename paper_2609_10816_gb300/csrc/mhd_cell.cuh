@@ -59,6 +59,24 @@ __device__ __forceinline__ void store_current(const Dev& D, const double* const*
   }
 }
 
+// A warp's running maximum of a grid's reduction (bit patterns of non-negative doubles order like the
+// values): raised to what the other warps have found so far (*out) before a pass over cells, and made
+// known to them after it, so that cells are soon judged against nearly the final maximum.
+__device__ __forceinline__ double warp_max_enter(double s, const unsigned long long* out) {
+  unsigned long long g = *(const volatile unsigned long long*)out;
+  g = __shfl_sync(0xffffffffu, g, 0);
+  return dfrom((long long)(g > (unsigned long long)dbits(s) ? g : (unsigned long long)dbits(s)));
+}
+__device__ __forceinline__ double warp_max_leave(double s, double entered, unsigned long long* out) {
+  unsigned long long b = (unsigned long long)dbits(s);
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long t = __shfl_xor_sync(0xffffffffu, b, o);
+    b = t > b ? t : b;
+  }
+  if ((threadIdx.x & 31) == 0 && b > (unsigned long long)dbits(entered)) atomicMax(out, b);
+  return dfrom((long long)b);
+}
+
 // ---- CFL signal speed (Sec. 2.4, Eq. waves:fast-speed) ----------------------------------------
 // max(m, s) for the cell's speed s = max_d (|u_d| + c_f,d) hmin / h_d, given a running maximum m.
 // With S = a^2 + b^2/rho, every fast speed lies between sqrt(max(a^2, b^2/rho)) and sqrt(S) (the
@@ -66,14 +84,61 @@ __device__ __forceinline__ void store_current(const Dev& D, const double* const*
 // so the three fast speeds are evaluated only when the upper bound, widened by 1e-12 against
 // rounding, reaches m: the running maximum is the same value, with no square root for most cells
 // of a cubic grid (one otherwise) instead of six. A non-finite speed gives +inf.
+// Most cells are settled before that in single precision: the cell's speed is certainly below m when
+// an upper bound of it, formed from the conserved values rounded to floats and widened by 2^-12
+// (every float operation is good to 2^-22, and p, the difference of energies, to 2^-18 of e_tot, which
+// is added to it), stays below m. The FP64 instructions of a cell take 35 x 64 cycles of their pipe,
+// these about 100 of others: 192^3 turbulence, mhd_max_dt and mhd_divb 0.60 ms, so 0.32.
+// Only states of ordinary size are judged (every value below 2^60, rho and e_tot positive and above
+// 2^-30, m above 2^-40, p certainly positive), so that nothing overflows, flushes to zero or is not a
+// number.
+__device__ __forceinline__ float to_float(double x) {  // for |x| < 2^60; below 2^-126: 0
+  const unsigned hi = (unsigned)__double2hiint(x), mag = hi & 0x7fffffffu;
+  const unsigned f = __funnelshift_l((unsigned)__double2loint(x), mag - (896u << 20), 3);
+  return __int_as_float(mag < (897u << 20) ? 0 : (int)(f | (hi & 0x80000000u)));
+}
+__device__ __forceinline__ bool cfl_below(const Dev& D, const double* u, const double* lo, const double* hi, double m) {
+  unsigned big = 0;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) big = max(big, (unsigned)__double2hiint(u[v]) & 0x7fffffffu);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    big = max(big, (unsigned)__double2hiint(lo[d]) & 0x7fffffffu);
+    big = max(big, (unsigned)__double2hiint(hi[d]) & 0x7fffffffu);
+  }
+  const int small = 993 << 20;  // 2^-30; a negative value's high word is below it too
+  if (big >= (1083u << 20) || min(__double2hiint(u[0]), __double2hiint(u[4])) < small ||
+      __double2hiint(m) < (983 << 20) || __double2hiint(m) >= (1083 << 20))
+    return false;
+  const float rho = to_float(u[0]), e = to_float(u[4]), gm1 = to_float(D.gm1), gam = to_float(D.gam);
+  float ri;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ri) : "f"(rho));
+  float um = 0.0f, u2 = 0.0f, b2 = 0.0f;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const float ud = to_float(u[1 + d]) * ri, bd = 0.5f * (to_float(lo[d]) + to_float(hi[d]));
+    um = fmaxf(um, fabsf(ud));
+    u2 = fmaf(ud, ud, u2);
+    b2 = fmaf(bd, bd, b2);
+  }
+  const float ei = e - 0.5f * fmaf(rho, u2, b2), err = e * 3.814697265625e-06f;  // 2^-18
+  if (!(ei > err)) return false;
+  const float s2 = fmaf(gam * gm1, ei + err, b2) * ri;
+  return (um + sqrtf(s2)) * 1.000244140625f < to_float(m);
+}
+
 __device__ __forceinline__ double cfl_speed_max(const Dev& D, const double* U, const double* const* B, long long X,
                                                 double m, double* Pout = nullptr) {
-  double w[8];
-  prim_of(D, U, B, X, w);
+  double w[8], u[5], blo[3], bhi[3];
+  load_cell(D, U, B, X, u, blo, bhi);
+  const bool below = cfl_below(D, u, blo, bhi, m);
+  if (!Pout && below) return m;
+  prim_from(D, u, blo, bhi, w);
   if (Pout) {  // the primitives of the state, for a stage that starts from it
 #pragma unroll
     for (int v = 0; v < 8; ++v) Pout[v * D.N + X] = w[v];
     store_current(D, B, X);
+    if (below) return m;
   }
   // a cell with a value that is not finite gives +inf, which the callers report as an error
   bool ok = true;
