@@ -318,13 +318,12 @@ __global__ void __launch_bounds__(128) k_adj_edges(AdjDev A) {
   const Dev& D = A.D;
   const long long X = aid();
   const long long N = D.N;
-  double etaacc = 0.0;
   const int e = blockIdx.y, a = (e + 1) % 3, c = (e + 2) % 3;
   constexpr int NE = EMF == EMF_FS18 ? 20 : (EMF == EMF_B25A ? 12 : 8);  // adjoint slots per edge
   const double lam = X < N ? A.lE[e * N + X] : 0.0;
   if (X < N && lam == 0.0)
     for (int k = 0; k < NE; ++k) A.lEdge[(NE * e + k) * N + X] = 0.0;
-  if (lam != 0.0) {  // no early return: the whole warp sums d/d(eta) below
+  if (lam != 0.0) {
     const long long Xc = shift(D, X, c, -1), Xa = shift(D, X, a, -1);
     // the reconstructed edge values as the forward edge sweeps formed them. Q26: b_a, u_a* bottom
     // and top (Epart), b_c, u_c* left and right (EdgeC). FS18: b_a bottom and top (Epart), b_c
@@ -385,19 +384,7 @@ __global__ void __launch_bounds__(128) k_adj_edges(AdjDev A) {
     atomicAdd(&A.lAm[a * N + (wa_m ? Xc : X)], g[NI - 3]);
     atomicAdd(&A.lAp[c * N + (wc_p ? Xa : X)], g[NI - 2]);
     atomicAdd(&A.lAm[c * N + (wc_m ? Xa : X)], g[NI - 1]);
-    if (D.resistive) {  // E += eta j, j = (b_c[X] - b_c[X-a]) / h_a - (b_a[X] - b_a[X-c]) / h_c
-      const double* Ba = D.Bin[a];
-      const double* Bc = D.Bin[c];
-      const double j = (Bc[X] - Bc[Xa]) * D.hinv[a] - (Ba[X] - Ba[Xc]) * D.hinv[c];
-      etaacc += lam * j;
-      const double la = D.eta * lam * D.hinv[a], lc = D.eta * lam * D.hinv[c];
-      atomicAdd(&A.lB[c * N + X], la);
-      atomicAdd(&A.lB[c * N + Xa], -la);
-      atomicAdd(&A.lB[a * N + X], -lc);
-      atomicAdd(&A.lB[a * N + Xc], lc);
-    }
   }
-  warp_add(etaacc, A.lEta);
 }
 
 // ---- edge reconstructions: adjoint of the face arrays reconstructed to the edges -----------
@@ -831,17 +818,56 @@ __device__ __forceinline__ double joule_adj(const AdjDev& A, int d, long long X,
 }
 
 
-__global__ void __launch_bounds__(128) k_adj_joule(AdjDev A) {
+// The resistive terms gathered, without atomics: E_e += eta j_e, and the Joule flux of a d-face
+// (a = d + 1, c = d + 2), eta / 2 (sa bcbar - sc babar) with sa = j_a[X] + j_a[X + c],
+// sc = j_c[X] + j_c[X + a] and bcbar, babar the means of the two cells' b_c, b_a.
+// Pass 1, per edge: j and the adjoint of eta j, W = lE + (sum over the four faces whose flux holds
+// it) / 2 into the edge adjoints' memory (free by now): rows 0-2 W, 3-5 j; d/d(eta) = sum W j.
+__device__ __forceinline__ double* adj_w(const AdjDev& A, int e) { return A.lEdge + e * A.D.N; }
+__device__ __forceinline__ double* adj_j(const AdjDev& A, int e) { return A.lEdge + (3 + e) * A.D.N; }
+__global__ void __launch_bounds__(128) k_adj_current(AdjDev A) {
   const Dev& D = A.D;
-  const int d = blockIdx.y;
-  if (!D.resistive) return;
-  const long long X = aid();
-  const long long N = D.N;
-  const double lam = X < N ? A.lF[(5LL * d + 4) * N + X] : 0.0;
+  const long long X = aid(), N = D.N;
+  const int e = blockIdx.y, a = (e + 1) % 3, c = (e + 2) % 3;
   double deta = 0.0;
-  if (lam != 0.0) deta = joule_adj(A, d, X, lam);
+  if (X < N) {
+    const long long Xa = shift(D, X, a, -1), Xc = shift(D, X, c, -1);
+    const double j = fma(D.Bin[c][X] - D.Bin[c][Xa], D.hinv[a], -((D.Bin[a][X] - D.Bin[a][Xc]) * D.hinv[c]));
+    // mean tangential field k of the d-face at Y, times twice the face's energy adjoint
+    auto lb = [&](int d, int k, long long Y) {
+      const double* b = D.P + (5 + k) * N;
+      return A.lF[(5LL * d + 4) * N + Y] * (b[shift(D, Y, d, -1)] + b[Y]);
+    };
+    // as j_a of the faces along d = e + 2 = c (their c is a): X and X - a; as j_c of those along
+    // d = e + 1 = a (their a is c): X and X - c
+    const double s = (lb(c, a, X) + lb(c, a, Xa)) - (lb(a, c, X) + lb(a, c, Xc));
+    const double w = fma(0.25, s, A.lE[e * N + X]);
+    adj_w(A, e)[X] = w;
+    adj_j(A, e)[X] = j;
+    deta = w * j;
+  }
   warp_add(deta, A.lEta);
 }
+// Pass 2, per cell and component k: the lower k-face's share of the four currents it enters, and the
+// cell's b_k's share of the Joule fluxes of the four faces around that hold it.
+__global__ void __launch_bounds__(128) k_adj_current_b(AdjDev A) {
+  const Dev& D = A.D;
+  const long long X = aid(), N = D.N;
+  if (X >= N) return;
+  const int k = blockIdx.y, p = (k + 1) % 3, q = (k + 2) % 3;
+  // j_p = d b_k / d q - ... (k = c of the p-edges), j_q = ... - d b_k / d p (k = a of the q-edges)
+  const double *wp = adj_w(A, p), *wq = adj_w(A, q), *jp = adj_j(A, p), *jq = adj_j(A, q);
+  const long long Xp = shift(D, X, p, 1), Xq = shift(D, X, q, 1);
+  A.lB[k * N + X] += D.eta * fma(wp[X] - wp[Xq], D.hinv[q], -((wq[X] - wq[Xp]) * D.hinv[p]));
+  // p-faces hold b_k as b_c with j_q as j_a: sa = j_q[Y] + j_q[Y + k]; q-faces as b_a with j_p as j_c:
+  // sc = j_p[Y] + j_p[Y + k]
+  auto term = [&](const double* j, int d, long long Y) {
+    return A.lF[(5LL * d + 4) * N + Y] * (j[Y] + j[shift(D, Y, k, 1)]);
+  };
+  const double t = (term(jq, p, X) + term(jq, p, Xp)) - (term(jp, q, X) + term(jp, q, Xq));
+  A.lP[(5 + k) * N + X] = fma(0.25 * D.eta, t, A.lP[(5 + k) * N + X]);
+}
+
 // ---- face reconstructions: adjoint of the primitives --------------------------------------
 // (one direction and variable per blockIdx.y)
 template <int RC>
@@ -1250,7 +1276,10 @@ static void adj_flux_r(const AdjDev& A, int rs, cudaStream_t st) {
   if (rs == RS_HLL) k_adj_faces<RC, RS_HLL><<<nb3, 128, 0, st>>>(A);
   else if (rs == RS_HLLD) k_adj_faces<RC, RS_HLLD><<<nb3, 128, 0, st>>>(A);
   else k_adj_faces<RC, RS_LLF><<<nb3, 128, 0, st>>>(A);
-  if (A.D.resistive) k_adj_joule<<<nb3, 128, 0, st>>>(A);
+  if (A.D.resistive) {
+    k_adj_current<<<nb3, 128, 0, st>>>(A);
+    k_adj_current_b<<<nb3, 128, 0, st>>>(A);
+  }
   if (RC == REC_PPM) rec_sweeps<1>(A, st);
   else k_adj_face_rec<RC><<<dim3(nb, 21), 128, 0, st>>>(A);
   k_adj_prim<<<nb, 128, 0, st>>>(A);
