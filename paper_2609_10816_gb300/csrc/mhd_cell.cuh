@@ -258,20 +258,6 @@ __device__ __forceinline__ bool invalid_vals(const Dev& D, const double* u, cons
   }
   return false;
 }
-__device__ __forceinline__ bool invalid_cell(const Dev& D, const double* U, double* const* B, long long X) {
-  const long long N = D.N;
-  double u[5], lo[3], hi[3];
-#pragma unroll
-  for (int v = 0; v < 5; ++v) u[v] = U[v * N + X];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    lo[d] = B[d][X];
-    hi[d] = B[d][shift(D, X, d, 1)];
-  }
-  return invalid_vals(D, u, lo, hi);
-}
-
-
 // invalid_vals and the primitives w of the same state in one pass: the pressure the test needs
 // is w[4], formed by the same operations (so the flag is the same bit for bit)
 __device__ __forceinline__ bool prim_invalid(const Dev& D, const double* u, const double* lo, const double* hi,

@@ -72,10 +72,6 @@ __device__ __forceinline__ bool is_zero(double x) { return mag_bits(x) == 0; }
 __device__ __forceinline__ bool same_sign(double a, double b) {
   return (gt0(a) && gt0(b)) || (lt0(a) && lt0(b));
 }
-// sgn(x) in {-1, 0, +1} as a double (bit construction, no FP64 op)
-__device__ __forceinline__ double sgnd(double x) {
-  return gt0(x) ? 1.0 : (lt0(x) ? -1.0 : 0.0);
-}
 __device__ __forceinline__ bool finite_d(double x) {
   return (mag_bits(x) >> 52) != 0x7ff;
 }
@@ -217,7 +213,6 @@ __device__ __forceinline__ bool ge0(const Dual& x) { return ge0(x.v); }
 __device__ __forceinline__ bool vgt(const Dual& a, const Dual& b) { return vgt(a.v, b.v); }
 __device__ __forceinline__ bool is_zero(const Dual& x) { return is_zero(x.v); }
 __device__ __forceinline__ bool same_sign(const Dual& a, const Dual& b) { return same_sign(a.v, b.v); }
-__device__ __forceinline__ double sgnd(const Dual& x) { return sgnd(x.v); }
 // |m| with the sign of s
 __device__ __forceinline__ Dual with_sign(Dual m, Dual s) {
   const bool flip = (dbits(m.v) < 0) != (dbits(s.v) < 0);
