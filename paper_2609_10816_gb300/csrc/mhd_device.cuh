@@ -370,7 +370,8 @@ __device__ __forceinline__ double vl_slope2(double dl, double dr) {
 enum { PPM_FLAT = 0, PPM_FIX_L = 1, PPM_FIX_R = 2, PPM_KEEP = 3 };
 // which constraint applies for s1 = aR - a, s2 = a - aL
 __device__ __forceinline__ int ppm_mono_case(double s1, double s2) {
-  const long long m1 = mag_bits(s1), m2 = mag_bits(s2), two = 1LL << 52;
+  // (unsigned: the doubling of an infinity or a NaN stays the larger)
+  const unsigned long long m1 = (unsigned long long)mag_bits(s1), m2 = (unsigned long long)mag_bits(s2), two = 1ULL << 52;
   if ((dbits(s1) ^ dbits(s2)) < 0 || m1 == 0 || m2 == 0) return PPM_FLAT;  // a is an extremum
   if (m2 > m1 + two) return PPM_FIX_L;                                     // aL = 3a - 2aR = a - 2 s1
   if (m2 + two < m1) return PPM_FIX_R;                                     // aR = 3a - 2aL = a + 2 s2
@@ -829,27 +830,40 @@ __device__ __forceinline__ void phys_speed(const FaceStateT<T>& s, T bn, double 
   phys_speed_a(s, bn * bn, gam, o);
   o.cf2 = halve(rcp(s.rho)) * o.A;
 }
-// Which side has the larger fast speed, decided on A_L rho_R against A_R rho_L (no quotient).
+// Which side has the larger fast speed, decided on A_L rho_R against A_R rho_L (no quotient); plain
+// tells whether both products and x = A rho / 2 of that side are positive normal numbers.
 template <class T>
 __device__ __forceinline__ bool fast_left(const FaceStateT<T>& sl, const FaceStateT<T>& sr, const PhysFluxT<T>& L,
-                                          const PhysFluxT<T>& R, bool& finite) {
+                                          const PhysFluxT<T>& R, T& ah, T& x, bool& plain) {
   const double tl = val(L.A) * val(sr.rho), tr = val(R.A) * val(sl.rho);
-  finite = finite_d(tl) && finite_d(tr);
-  return dbits(tl) >= dbits(tr);
+  const bool left = dbits(tl) >= dbits(tr);
+  ah = halve(left ? L.A : R.A);
+  x = ah * (left ? sl.rho : sr.rho);
+  const unsigned a = (unsigned)__double2hiint(tl) - 0x00100000u, b = (unsigned)__double2hiint(tr) - 0x00100000u,
+                 c = (unsigned)__double2hiint(val(x)) - 0x00100000u;
+  plain = max(max(a, b), c) < 0x7fe00000u;
+  return left;
+}
+// The same for states whose products under- or overflow, a density or pressure below zero, infinities
+// and NaN (not inlined: see the reciprocals): the larger of the quotients A / (2 rho), which for a
+// negative density loses against the other side's.
+template <class T>
+__device__ __noinline__ T fast_max_any(T rl, T rr, T Al, T Ar, bool& left) {
+  const T cl = halve(rcp(rl)) * Al, cr = halve(rcp(rr)) * Ar;
+  left = dbits(val(cl)) >= dbits(val(cr));
+  return sqrt_(left ? cl : cr);
 }
 // The larger of the two fast speeds, sqrt(A / (2 rho)) of that side = (A/2) / sqrt(rho A/2): one
 // reciprocal square root in the place of two reciprocals and a square root (9 FP64 instructions
-// against 14). A state that is not finite on either side gives a speed that is not a number.
+// against 14).
 template <class T>
 __device__ __forceinline__ T fast_max(const FaceStateT<T>& sl, const FaceStateT<T>& sr, const PhysFluxT<T>& L,
                                       const PhysFluxT<T>& R) {
-  bool fin;
-  const bool left = fast_left(sl, sr, L, R, fin);
-  const T ah = halve(left ? L.A : R.A);
-  const T x = ah * (left ? sl.rho : sr.rho);
-  const T c = vabs(ah) * rsqrt_(x);
-  if (!fin) return T(dfrom(0x7ff8000000000000LL));
-  return is_zero(x) ? T(0.0) : c;
+  bool plain;
+  T ah, x;
+  bool left = fast_left(sl, sr, L, R, ah, x, plain);
+  if (!plain) return fast_max_any(sl.rho, sr.rho, L.A, R.A, left);
+  return vabs(ah) * rsqrt_(x);
 }
 
 // Conserved vector and ideal-MHD flux of Eq. (mhd:conservation-laws) in the face frame, with e_tot

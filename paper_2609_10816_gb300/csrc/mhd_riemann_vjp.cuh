@@ -357,14 +357,18 @@ __device__ __forceinline__ void riemann_vjp(const FaceState& sl, const FaceState
   } else {
     phys_speed_a(sl, bn2, gam, L);
     phys_speed_a(sr, bn2, gam, R);
-    bool fin;
-    cmax_left = fast_left(sl, sr, L, R, fin);
+    bool plain;
+    double ah, x, cmax;
+    cmax_left = fast_left(sl, sr, L, R, ah, x, plain);
     // fast_max, and 1 / c from the same reciprocal root (0 where c is 0)
-    const double ah = halve(cmax_left ? L.A : R.A), rc = cmax_left ? sl.rho : sr.rho, x = ah * rc;
-    const double y = rsqrt_(x);
-    const bool z = is_zero(x);
-    const double cmax = !fin ? dfrom(0x7ff8000000000000LL) : (z ? 0.0 : vabs(ah) * y);
-    icmax = z ? 0.0 : rc * y;
+    if (plain) {
+      const double y = rsqrt_(x);
+      cmax = vabs(ah) * y;
+      icmax = vabs(cmax_left ? sl.rho : sr.rho) * y;
+    } else {
+      cmax = fast_max_any(sl.rho, sr.rho, L.A, R.A, cmax_left);
+      icmax = is_zero(cmax) ? 0.0 : rcp(cmax);
+    }
     umax_left = okey(sl.u) >= okey(sr.u);
     umin_left = okey(sl.u) <= okey(sr.u);
     const double umax = umax_left ? sl.u : sr.u, umin = umin_left ? sl.u : sr.u;
