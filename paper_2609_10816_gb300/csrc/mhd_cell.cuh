@@ -85,9 +85,12 @@ __device__ __forceinline__ double warp_max_leave(double s, double entered, unsig
 // rounding, reaches m: the running maximum is the same value, with no square root for most cells
 // of a cubic grid (one otherwise) instead of six. A non-finite speed gives +inf.
 // Most cells are settled before that in single precision: the cell's speed is certainly below m when
-// an upper bound of it, formed from the conserved values rounded to floats and widened by 2^-12
-// (every float operation is good to 2^-22, and p, the difference of energies, to 2^-18 of e_tot, which
-// is added to it), stays below m. The FP64 instructions of a cell take 35 x 64 cycles of their pipe,
+// an upper bound of it, formed from the conserved values cut to floats and widened by 2^-12, stays
+// below m. Every product, sum of squares and root is good to 2^-20 of itself; the two differences are
+// not, and carry bounds of their own: p, the difference of energies, takes 2^-18 of e_tot more, and the
+// mean of two face values b, which may cancel (a field that alternates from face to face), lies within
+// 2^-23 (|lo| + |hi|) of its float, so that b^2 is taken at the upper end of that interval where it adds
+// to the speed and at the lower end where it takes from p. The FP64 instructions of a cell take 35 x 64 cycles of their pipe,
 // these about 100 of others: 192^3 turbulence, mhd_max_dt and mhd_divb 0.60 ms, so 0.32.
 // Only states of ordinary size are judged (every value below 2^60, rho and e_tot positive and above
 // 2^-30, m above 2^-40, p certainly positive), so that nothing overflows, flushes to zero or is not a
@@ -113,17 +116,20 @@ __device__ __forceinline__ bool cfl_below(const Dev& D, const double* u, const d
   const float rho = to_float(u[0]), e = to_float(u[4]), gm1 = to_float(D.gm1), gam = to_float(D.gam);
   float ri;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ri) : "f"(rho));
-  float um = 0.0f, u2 = 0.0f, b2 = 0.0f;
+  float um = 0.0f, u2 = 0.0f, b2 = 0.0f, b2lo = 0.0f;  // b2lo <= b^2 <= b2
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const float ud = to_float(u[1 + d]) * ri, bd = 0.5f * (to_float(lo[d]) + to_float(hi[d]));
+    const float ud = to_float(u[1 + d]) * ri, fl = to_float(lo[d]), fh = to_float(hi[d]);
+    const float bd = fabsf(0.5f * (fl + fh)), off = 1.1920928955078125e-07f * (fabsf(fl) + fabsf(fh));  // 2^-23
+    const float bmax = bd + off, bmin = fmaxf(bd - off, 0.0f);
     um = fmaxf(um, fabsf(ud));
     u2 = fmaf(ud, ud, u2);
-    b2 = fmaf(bd, bd, b2);
+    b2 = fmaf(bmax, bmax, b2);
+    b2lo = fmaf(bmin, bmin, b2lo);
   }
-  const float ei = e - 0.5f * fmaf(rho, u2, b2), err = e * 3.814697265625e-06f;  // 2^-18
-  if (!(ei > err)) return false;
-  const float s2 = fmaf(gam * gm1, ei + err, b2) * ri;
+  const float err = e * 3.814697265625e-06f;  // 2^-18
+  if (!(e - 0.5f * fmaf(rho, u2, b2) > err)) return false;
+  const float s2 = fmaf(gam * gm1, e - 0.5f * fmaf(rho, u2, b2lo) + err, b2) * ri;
   return (um + sqrtf(s2)) * 1.000244140625f < to_float(m);
 }
 
