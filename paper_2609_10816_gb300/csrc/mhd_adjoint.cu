@@ -60,7 +60,8 @@ __device__ __forceinline__ void half_slope_jac(double dl, double dr, double& gl,
   if (dbits(m) <= dbits(0.25 * vabs(dl + dr))) (left_min ? gl : gr) = 1.0;
   else { gl = 0.25; gr = 0.25; }
 }
-template <int R>
+// FACE: the values are a face sweep's (PPM-EP forms its offsets there in fixed point).
+template <int R, bool FACE>
 __device__ __forceinline__ void recon_jac(const double* q, double* JL, double* JR) {
 #pragma unroll
   for (int k = 0; k < 5; ++k) JL[k] = JR[k] = 0.0;
@@ -73,15 +74,15 @@ __device__ __forceinline__ void recon_jac(const double* q, double* JL, double* J
     JL[1] = -h1; JL[2] = 1.0 - h2; JL[3] = -h3;
     JR[1] = h1;  JR[2] = 1.0 + h2; JR[3] = h3;
   } else if (R == REC_PPM_EP) {
-    // the decisions of Rec<REC_PPM_EP> on the same window
+    // the decisions of Rec<REC_PPM_EP> on the same window, from values formed the same way
     const double e0 = q[1] - q[0], e1 = q[2] - q[1], e2 = q[3] - q[2], e3 = q[4] - q[3];
     const int s0 = sgn_code(e0), s1 = sgn_code(e1), s2 = sgn_code(e2), s3 = sgn_code(e3);
     const int ka = cmp_code(e1, e0), kb = cmp_code(e2, e1), kc = cmp_code(e3, e2);
     const bool xa = ext_code(s0, s1, s2), xb = ext_code(s1, s2, s3);
     int pa, pb;  // 0: fourth-order value, 1: the lower cell's value, 2: the upper cell's
     double ra, sa, rb, sb;
-    ppm_ep_face<false>(q[1], q[2], e0, e1, e2, xa && same_code(ka, kb), pa, ra, sa);
-    ppm_ep_face<false>(q[2], q[3], e1, e2, e3, xb && same_code(kb, kc), pb, rb, sb);
+    ppm_ep_face<FACE>(q[1], q[2], e0, e1, e2, xa && same_code(ka, kb), pa, ra, sa);
+    ppm_ep_face<FACE>(q[2], q[3], e1, e2, e3, xb && same_code(kb, kc), pb, rb, sb);
     if (pa == 0) {
       JL[0] = -1.0 / 12.0; JL[1] = 7.0 / 12.0; JL[2] = 7.0 / 12.0; JL[3] = -1.0 / 12.0;
     } else {
@@ -150,7 +151,7 @@ __device__ __forceinline__ void recon_jac(const double* q, double* JL, double* J
 // adjoint of the reconstruction of `arr` along dir at point X: lam_lo / lam_hi are the adjoints of
 // its lower / upper values; the contributions go to the window's points (atomics: every point
 // gets them from the five windows it lies in, and more than once on lines shorter than five)
-template <int RC>
+template <int RC, bool FACE>
 __device__ __forceinline__ void rec_scatter(const Dev& D, const double* arr, long long X, int dir, double lam_lo,
                                             double lam_hi, double* out) {
   if (lam_lo == 0.0 && lam_hi == 0.0) return;
@@ -161,7 +162,7 @@ __device__ __forceinline__ void rec_scatter(const Dev& D, const double* arr, lon
     Z[k] = shift2(D, X, dir, k - 2);
     q[k] = arr[Z[k]];
   }
-  recon_jac<RC>(q, JL, JR);
+  recon_jac<RC, FACE>(q, JL, JR);
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     const double c = fma(JL[k], lam_lo, JR[k] * lam_hi);
@@ -445,7 +446,7 @@ __global__ void __launch_bounds__(128) k_adj_edge_rec(AdjDev A) {
     q = D.LR + row;
     out = A.lLR + row;
   }
-  rec_scatter<RC>(D, q, X, t, L[hi * N + X], L[(hi - 1) * N + Xt], out);
+  rec_scatter<RC, false>(D, q, X, t, L[hi * N + X], L[(hi - 1) * N + Xt], out);
 }
 
 // ---- reconstructions as reverse sweeps (PPM) ------------------------------------------------
@@ -882,7 +883,7 @@ __global__ void __launch_bounds__(128) k_adj_face_rec(AdjDev A) {
   const double* lLR = A.lLR + 14LL * dir * N;
   const long long Xn = shift(D, X, dir, 1);
   // point X's lower value = right state of face X, upper value = left state of face X + dir
-  rec_scatter<RC>(D, D.P + slot * N, X, dir, lLR[(7 + v) * N + X], lLR[v * N + Xn], A.lP + slot * N);
+  rec_scatter<RC, true>(D, D.P + slot * N, X, dir, lLR[(7 + v) * N + X], lLR[v * N + Xn], A.lP + slot * N);
 }
 
 // ---- primitives: adjoint of cons -> prim ------------------------------------------------
@@ -1224,8 +1225,8 @@ __global__ void __launch_bounds__(128) k_adj_eps_rec(AdjDev A) {
     const int a = (e + 1) % 3, c = (e + 2) % 3;
     const double* lfL = A.lEf + 2LL * e * N;
     const double* lfB = A.lEf + 6 * N + 2LL * e * N;
-    rec_scatter<RC>(D, A.eps + e * N, X, a, lfL[N + X], lfL[shift(D, X, a, 1)], A.leps + e * N);
-    rec_scatter<RC>(D, A.eps + e * N, X, c, lfB[N + X], lfB[shift(D, X, c, 1)], A.leps + e * N);
+    rec_scatter<RC, false>(D, A.eps + e * N, X, a, lfL[N + X], lfL[shift(D, X, a, 1)], A.leps + e * N);
+    rec_scatter<RC, false>(D, A.eps + e * N, X, c, lfB[N + X], lfB[shift(D, X, c, 1)], A.leps + e * N);
   }
 }
 // the cell EMF's adjoint into the primitives' (one thread per cell, no other writer meanwhile)
