@@ -808,6 +808,8 @@ using PhysFlux = PhysFluxT<double>;
 // a + b with no product fused into it: the larger-speed decision (fast_left) compares the two sides,
 // and equal states have to tie however the code around them is compiled
 __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+// a b that is not fused into a sum it enters
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ Dual add_rn(Dual a, Dual b) { return Dual(__dadd_rn(a.v, b.v), a.t + b.t); }
 
 // Total pressure and the fast magnetosonic speed of Eq. (waves:fast-speed) along the normal, as

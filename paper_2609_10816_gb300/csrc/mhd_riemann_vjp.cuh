@@ -3,11 +3,14 @@
 //
 // For weights (lf, lap, lam, lus) the scalar g = sum_v lf[v] F[v] + lap alpha+ + lam alpha- +
 // lus u* of one face is differentiated with respect to the 15 inputs (left and right face states
-// and the normal field) in one reverse sweep. The forward values are recomputed with the same
-// device functions (phys_speed, phys_flux, star_state) in double precision, so every branch --
-// the max/min of the wave speeds, the HLLD fan region, the degenerate star state, the clamped
-// discriminant -- is the one the forward step took, and the derivative is the one of that branch
-// (ties and zero square roots as in the forward-mode dual numbers). Each reverse statement is
+// and the normal field) in one reverse sweep. The forward values that decide a branch are recomputed
+// with the same device functions (phys_speed, phys_flux, star_state) and the same roundings: the
+// forward kernels are compiled without contraction, this file's with it, so a product that enters
+// a sum on the way to a decision is a mul_rn here. Every branch -- the max/min of the wave speeds,
+// the HLLD fan region, the side of the contact, the degenerate star state, the clamped discriminant
+// -- is then the one the forward step took, also where two meet to rounding (a head-on collision of
+// equal gases), and the derivative is the one of that branch (ties and zero square roots as in the
+// forward-mode dual numbers). Each reverse statement is
 // the transpose of one forward statement, in reverse order.
 #pragma once
 #include "mhd_device.cuh"
@@ -146,8 +149,8 @@ __device__ __forceinline__ void hlld_rev(const FaceState& sl, const FaceState& s
   if (fan) {
     suL = SL - sl.u;
     suR = SR - sr.u;
-    mL = suL * sl.rho;
-    mR = suR * sr.rho;
+    mL = mul_rn(suL, sl.rho);
+    mR = mul_rn(suR, sr.rho);
     dinv = rcp(mR - mL);
     du = sr.u - sl.u;
     dpt = L.pt - R.pt;
@@ -175,7 +178,7 @@ __device__ __forceinline__ void hlld_rev(const FaceState& sl, const FaceState& s
     su = left ? suL : suR;
     m = left ? mL : mR;
     nS = left ? nL : fma(mL, du, dpt);
-    d = nS * dinv;
+    d = mul_rn(nS, dinv);
     pt = fma(m, d, qpt);
     ssm = su - d;
     star_state(q, m, su, d, ssm, bn, bn2, ssminv, a);
@@ -363,7 +366,7 @@ __device__ __forceinline__ void riemann_vjp(const FaceState& sl, const FaceState
     // fast_max, and 1 / c from the same reciprocal root (0 where c is 0)
     if (plain) {
       const double y = rsqrt_(x);
-      cmax = vabs(ah) * y;
+      cmax = mul_rn(vabs(ah), y);
       icmax = vabs(cmax_left ? sl.rho : sr.rho) * y;
     } else {
       cmax = fast_max_any(sl.rho, sr.rho, L.A, R.A, cmax_left);
