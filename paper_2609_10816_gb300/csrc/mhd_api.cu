@@ -141,6 +141,7 @@ void run_stage(mhd_ctx* c, const mhd::Dev& D, const Decoded& sc, PrimSource prim
     Timed t(c, MHD_K_FOFC, sc.fofc ? 2 : 1);
     if (sc.fofc) mhd::launch_fofc_fluxes(D, st);
     if (finish) {
+      if (cudaPeekAtLastError() != cudaSuccess) return;  // the caller reports it; the state stays as it was
       double* const b[3] = {finish->b0, finish->b1, finish->b2};
       mhd::launch_finish(D, sc.fofc, finish->cons, b, st);
     } else {

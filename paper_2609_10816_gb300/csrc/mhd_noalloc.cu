@@ -155,6 +155,7 @@ extern "C" mhd_status mhd_step_noalloc(const mhd_config* cfg, const mhd_state* s
     mhd::launch_flag(D, st);
     if (fofc) mhd::launch_fofc_fluxes(D, st);
     if (stage == 1) {
+      if (cudaPeekAtLastError() != cudaSuccess) break;  // reported below; the state stays as it was
       double* const b[3] = {state->b0, state->b1, state->b2};
       mhd::launch_finish(D, fofc, state->cons, b, st);
     } else if (fofc) {
