@@ -33,6 +33,15 @@ __device__ __forceinline__ void warp_add(double v, double* out) {
   if ((threadIdx.x & 31) == 0 && v != 0.0) atomicAdd(out, v);
 }
 
+// the same over a block of 128 threads (each of them calls it)
+__device__ __forceinline__ void block_add(double v, double* out) {
+  __shared__ double part[4];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) atomicAdd(out, (part[0] + part[1]) + (part[2] + part[3]));
+}
+
 // Jacobian of a point's reconstructed lower / upper values (aL, aR) in its window q[0..4]
 // (q[2] the point): every reconstruction is piecewise linear, so the rows follow from the branch
 // decisions, taken on the same values and with the same tie rules as the forward sweep.
@@ -823,14 +832,13 @@ __device__ __forceinline__ double joule_adj(const AdjDev& A, int d, long long X,
 // (a = d + 1, c = d + 2), eta / 2 (sa bcbar - sc babar) with sa = j_a[X] + j_a[X + c],
 // sc = j_c[X] + j_c[X + a] and bcbar, babar the means of the two cells' b_c, b_a.
 // Pass 1, per edge: j and the adjoint of eta j, W = lE + (sum over the four faces whose flux holds
-// it) / 2 into the edge adjoints' memory (free by now): rows 0-2 W, 3-5 j; d/d(eta) = sum W j.
+// it) / 2 into the edge adjoints' memory (free by now): rows 0-2 W, 3-5 j.
 __device__ __forceinline__ double* adj_w(const AdjDev& A, int e) { return A.lEdge + e * A.D.N; }
 __device__ __forceinline__ double* adj_j(const AdjDev& A, int e) { return A.lEdge + (3 + e) * A.D.N; }
 __global__ void __launch_bounds__(128) k_adj_current(AdjDev A) {
   const Dev& D = A.D;
   const long long X = aid(), N = D.N;
   const int e = blockIdx.y, a = (e + 1) % 3, c = (e + 2) % 3;
-  double deta = 0.0;
   if (X < N) {
     const long long Xa = shift(D, X, a, -1), Xc = shift(D, X, c, -1);
     const double j = fma(D.Bin[c][X] - D.Bin[c][Xa], D.hinv[a], -((D.Bin[a][X] - D.Bin[a][Xc]) * D.hinv[c]));
@@ -842,18 +850,25 @@ __global__ void __launch_bounds__(128) k_adj_current(AdjDev A) {
     // as j_a of the faces along d = e + 2 = c (their c is a): X and X - a; as j_c of those along
     // d = e + 1 = a (their a is c): X and X - c
     const double s = (lb(c, a, X) + lb(c, a, Xa)) - (lb(a, c, X) + lb(a, c, Xc));
-    const double w = fma(0.25, s, A.lE[e * N + X]);
-    adj_w(A, e)[X] = w;
+    adj_w(A, e)[X] = fma(0.25, s, A.lE[e * N + X]);
     adj_j(A, e)[X] = j;
-    deta = w * j;
   }
-  warp_add(deta, A.lEta);
 }
 // Pass 2, per cell and component k: the lower k-face's share of the four currents it enters, and the
-// cell's b_k's share of the Joule fluxes of the four faces around that hold it.
+// cell's b_k's share of the Joule fluxes of the four faces around that hold it. And d/d(eta) = sum W j,
+// summed over the cell's edges, then over the block: every addition to the running sum rounds its last
+// bit, so there are as few as blocks, and they meet after the components' terms have cancelled (64^3,
+// terms of +67 and -67 from the x and y edges: off by 4e-15; by 1.4e-12 with an addition per warp and
+// component). The 64^3 step takes 3.69 ms, with those 3.72.
 __global__ void __launch_bounds__(128) k_adj_current_b(AdjDev A) {
   const Dev& D = A.D;
   const long long X = aid(), N = D.N;
+  if (blockIdx.y == 0) {  // (uniform over the block)
+    double deta = 0.0;
+    if (X < N)
+      deta = fma(adj_w(A, 0)[X], adj_j(A, 0)[X], fma(adj_w(A, 1)[X], adj_j(A, 1)[X], adj_w(A, 2)[X] * adj_j(A, 2)[X]));
+    block_add(deta, A.lEta);
+  }
   if (X >= N) return;
   const int k = blockIdx.y, p = (k + 1) % 3, q = (k + 2) % 3;
   // j_p = d b_k / d q - ... (k = c of the p-edges), j_q = ... - d b_k / d p (k = a of the q-edges)
