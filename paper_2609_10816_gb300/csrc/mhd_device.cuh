@@ -626,22 +626,24 @@ __device__ __forceinline__ double ppm_ep_face(double qa, double qb, double dl, d
   return pick == 0 ? f : (pick == 1 ? qa : qb);
 }
 // sign code of a - b: a comparison (the rounded difference of two doubles has the sign of the exact
-// one)
+// one). Where a or b is not a number the difference is that NaN, with its sign: a NaN in b compares as
+// far on the other side of everything.
 __device__ __forceinline__ int cmp_code(double a, double b) {
-  const long long ka = okey(a), kb = okey(b);
+  const long long ka = okey(a), k = okey(b);
+  const long long kb = (hi_word(b) & 0x7fffffffu) > 0x7ff00000u ? ~k : k;
   const bool z = is_zero(a) && is_zero(b);  // +0 and -0 are equal
   return z ? 0 : ((int)(ka > kb) | ((int)(ka < kb) << 1));
 }
 
 template <> struct Rec<REC_PPM_EP> {
-  static constexpr int LB = 3, LA = 2, NS = 7, NB = 3;
+  static constexpr int LB = 3, LA = 2, NS = 7, NB = 4;
   double q1, q2;      // q[m], q[m+1]
   double dl, dq;      // q[m] - q[m-1], q[m+1] - q[m]
   double s2;          // q[m] - f1
   double f1;          // interface value at m - 1/2
   double aRprev;      // upper value of point m-1
-  int code;           // bits 0-1: sign code of the curvature of point m-1; bit 2: interface m - 1/2
-                      // lies at an extremum
+  int code;           // bits 0-1: sign code of the curvature of point m; bit 2: it is that of point m-1
+                      // too, and not 0; bit 3: interface m - 1/2 lies at an extremum
   template <class F> __device__ __forceinline__ void each(F f) {
     f(0, q1);
     f(1, q2);
@@ -670,19 +672,19 @@ template <> struct Rec<REC_PPM_EP> {
     dl = e2;
     dq = e3;
     f1 = fb;
-    code = kb | ((int)xb << 2);
+    code = kc | ((int)same_code(kb, kc) << 2) | ((int)xb << 3);
   }
   template <bool FACE>
   __device__ __forceinline__ void step(double qn, double& L, double& R) {
     const double dn = qn - q2;  // q[m+2] - q[m+1]
-    const int c0 = code & 3, c1 = cmp_code(dq, dl), cn = cmp_code(dn, dq);  // points m-1, m, m+1
-    const bool x1 = code >> 2;
+    const int c1 = code & 3, cn = cmp_code(dn, dq);  // points m, m+1
+    const bool same01 = code & 4, x1 = code & 8, same1n = same_code(c1, cn);
     const bool x2 = ext_code(sgn_code(dl), sgn_code(dq), sgn_code(dn));
     int p;
     double r, s;
-    const double f2 = ppm_ep_face<FACE>(q1, q2, dl, dq, dn, x2 && same_code(c1, cn), p, r, s);  // m + 1/2
+    const double f2 = ppm_ep_face<FACE>(q1, q2, dl, dq, dn, x2 && same1n, p, r, s);  // m + 1/2
     double aL = f1, aR = f2;
-    if (!((x1 || x2) && same_code(c0, c1) && same_code(c1, cn))) ppm_mono(q1, r, s2, aL, aR);
+    if (!((x1 || x2) && same01 && same1n)) ppm_mono(q1, r, s2, aL, aR);
     L = aRprev;
     R = aL;
     aRprev = aR;
@@ -692,7 +694,7 @@ template <> struct Rec<REC_PPM_EP> {
     dq = dn;
     s2 = s;
     f1 = f2;
-    code = c1 | ((int)x2 << 2);
+    code = cn | ((int)same1n << 2) | ((int)x2 << 3);
   }
 };
 
@@ -763,22 +765,21 @@ template <> struct LaneRec<REC_PPM> {
   }
 };
 template <> struct LaneRec<REC_PPM_EP> {
-  static constexpr int NP = 4, FIRST = 0, NQ = 3, NB = 3;
+  static constexpr int NP = 4, FIRST = 0, NQ = 3, NB = 4;
   __device__ __forceinline__ static void step(const LaneWalk& w, const double* q, double* prev, int& code, double& L,
                                               double& R) {
     const double dn = q[2] - q[1];
     const double dq = w.up1(dn, prev[0]), dl = w.up2(dn, prev[0]);
     const int c1 = cmp_code(dq, dl), cn = cmp_code(dn, dq);  // curvatures of points m, m + 1
-    const bool x2 = ext_code(sgn_code(dl), sgn_code(dq), sgn_code(dn));
+    const bool x2 = ext_code(sgn_code(dl), sgn_code(dq), sgn_code(dn)), same1n = same_code(c1, cn);
     int p;
     double r, s;
-    const double f2 = ppm_ep_face<true>(q[0], q[1], dl, dq, dn, x2 && same_code(c1, cn), p, r, s);
+    const double f2 = ppm_ep_face<true>(q[0], q[1], dl, dq, dn, x2 && same1n, p, r, s);
     const double s2 = w.up1(s, prev[1]);
     double aL = w.up1(f2, prev[2]), aR = f2;
-    const int mine = c1 | ((int)x2 << 2), before = w.up1(mine, code);
-    const int c0 = before & 3;
-    const bool x1 = before >> 2;
-    if (!((x1 || x2) && same_code(c0, c1) && same_code(c1, cn))) ppm_mono(q[0], r, s2, aL, aR);
+    const int mine = (int)same1n | ((int)x2 << 1), before = w.up1(mine, code);
+    const bool same01 = before & 1, x1 = before & 2;
+    if (!((x1 || x2) && same01 && same1n)) ppm_mono(q[0], r, s2, aL, aR);
     L = w.up1(aR, prev[3]);
     R = aL;
     prev[0] = dn;
