@@ -164,14 +164,16 @@ mhd_status mhd_step_adjoint(mhd_ctx *ctx, const mhd_state *state, const mhd_stat
                             double eta, double *dL_deta);
 
 /* Self-check of the arithmetic the kernels use in place of FP64 instructions: on n pseudo-random
- * positive inputs spread over [2^-40, 2^40], max_rel_err[0..2] receive the largest relative
- * differences of the reciprocal, reciprocal square root and square root (hardware approximation +
- * one third-order Newton correction) from CUDA's IEEE 1/x, 1/sqrt(x) and sqrt(x); on n raw bit
+ * inputs (spread over [2^-40, 2^40], over every normal binade, over the first and last of them, and
+ * next to powers of two; reciprocals of either sign where they are normal), max_rel_err[0..2] receive
+ * the largest relative differences of the reciprocal, reciprocal square root and square root (a seed of
+ * about 30 bits + one Newton correction) from CUDA's IEEE 1/x, 1/sqrt(x) and sqrt(x); on n raw bit
  * patterns (subnormal, smallest, largest and non-finite binades among them), max_rel_err[3] and
  * [4] receive how many times the integer-pipe halving and quadrupling differ in any bit from the
  * FP64 multiplies by 0.5 and 4, and max_rel_err[5] on n pairs of non-NaN doubles (zeros,
  * subnormals, extreme binades and infinities among them) how many times an integer-pipe sign
- * test, comparison, min/max, |x|, sign copy or sign flip disagrees with the IEEE operation;
+ * test, comparison, min/max, |x|, sign copy or sign flip disagrees with the IEEE operation, or a root of
+ * a negative number or a zero is not NaN or 0;
  * max_rel_err[6] on n pairs (nearby and extreme exponents, few significand bits for exact
  * products and ties, any bit pattern, small integers and zeros) how many times the integer-pipe
  * multiply of mhd_fp64_rate's kinds 4-6 differs in any bit from the FP64 multiply (0 expected

@@ -152,7 +152,10 @@ __global__ void __launch_bounds__(256) k_divb(Dev D, Ptr3 Bp, unsigned long long
   block_max_atomic(mb, out + 1);
 }
 
-// relative error of rcp / rsqrt_ / sqrt_ against IEEE division and sqrt on hashed inputs
+// relative error of rcp / rsqrt_ / sqrt_ against IEEE division and sqrt on hashed inputs: in turn exponents
+// around 1, any, the ends of the range (where the seeds' exponent arithmetic and the general forms
+// take over from each other), and significands next to 1 and 2; reciprocals of either sign, where the
+// result is normal
 __global__ void __launch_bounds__(256) k_math_check(long long n, unsigned long long* out) {
   const long long i = cell_id();
   double er = 0.0, es = 0.0, eq = 0.0;
@@ -161,13 +164,23 @@ __global__ void __launch_bounds__(256) k_math_check(long long n, unsigned long l
     z ^= z >> 31;
     z *= 0xBF58476D1CE4E5B9ull;
     z ^= z >> 29;
-    const long long mant = (long long)(z & 0x000fffffffffffffull);
-    const long long ex = 1023 - 40 + (long long)((z >> 52) % 81);
-    const double x = dfrom((ex << 52) | mant);
-    const double r0 = 1.0 / x, s0 = sqrt(x), q0 = 1.0 / s0;
-    er = vabs(rcp(x) - r0) / r0;
+    long long mant = (long long)(z & 0x000fffffffffffffull);
+    long long ex = 1023 - 40 + (long long)((z >> 52) % 81);
+    const unsigned h = (unsigned)(z >> 32) * 0x85EBCA6Bu >> 8;
+    if ((i & 3) == 1) ex = 1 + (long long)(h % 2046u);
+    if ((i & 3) == 2) ex = (h & 8) ? 2046 - (long long)(h & 7) : 1 + (long long)(h & 7);
+    if ((i & 3) == 3) {
+      mant = (h & 1) ? mant & 0xffll : 0x000fffffffffffffll - (mant & 0xffll);
+      ex = 1 + (long long)((h >> 1) % 2046u);
+    }
+    const double x = dfrom((ex << 52) | mant), xs = neg_if((h >> 12) & 1, x);
+    const double r0 = 1.0 / xs, s0 = sqrt(x), q0 = 1.0 / s0;
+    if (mag_bits(r0) >= (1LL << 52)) er = vabs((rcp(xs) - r0) / r0);
     es = vabs(rsqrt_(x) - q0) / q0;
     eq = vabs(sqrt_(x) - s0) / s0;
+    // roots of zeros and of negative numbers
+    const double g = sqrt_(neg_if(true, x)), y = rsqrt_(neg_if(true, x));
+    if (g == g || y == y || sqrt_(neg_if(i & 1, 0.0)) != 0.0) atomicAdd(out + 5, 1ull);
   }
   block_max_atomic(er, out);
   block_max_atomic(es, out + 1);
