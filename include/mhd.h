@@ -184,7 +184,7 @@ mhd_status mhd_math_check(mhd_ctx *ctx, long long n, double *max_rel_err);
 /* Measured rate of one FP64 instruction kind on the current GPU (the pipe that bounds every
  * kernel of the step, hence the denominator of its roofline; the paper has no counterpart):
  * kind 0 DFMA, 1 DADD, 2 DMUL, 3 FP32 FFMA for comparison. Independent chains (eight per
- * thread, 8 blocks of 256 threads per SM) run `iters` steps each, timed with CUDA events on
+ * thread, operands in registers, 8 blocks of 256 threads per SM) run `iters` steps each, timed with CUDA events on
  * `cuda_stream` after a shorter warm-up; *ops_per_s receives instructions per second (per
  * thread-lane). Kinds 4-6 measure a binary64 multiply done on the integer pipe (bit for bit the
  * FP64 multiply; mhd_math_check verifies it) that the step's kernels do not use: 4 eight chains

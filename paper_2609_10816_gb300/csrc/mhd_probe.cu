@@ -6,7 +6,10 @@
 // pipe's throughput. The probe runs independent chains of one instruction kind (eight chains per
 // thread, enough to hide the pipe's latency) over a grid of 8 blocks of 256 threads per SM and
 // times them with CUDA events on the context's stream. The chains stay bounded (x <- a x + b with
-// 0 < a < 1), and their sum is stored so that nothing is optimised away. Kinds 4-6 run chains of
+// 0 < a < 1), and their sum is stored so that nothing is optimised away. The constants a, b differ from
+// thread to thread, so that they sit in registers as the operands of the step's kernels mostly do: with an
+// operand from the constant bank a DFMA takes 76 cycles of its pipe for a warp, as an add or a multiply
+// does anyway, with registers alone 64. Kinds 4-6 run chains of
 // the integer-pipe multiply (mhd_softmul.cuh), alone and mixed with DFMA chains, at the probe's
 // occupancy and at the face sweep's (2 blocks of 128 threads per SM). Kinds 7 and 8 run the DFMA
 // chains on 16 and 8 lanes of every warp (the others exit at once): whether the pipe's throughput
@@ -25,8 +28,9 @@ constexpr int kChains = 8;
 // integer-pipe multiply and NF chains of DFMA; KIND 5: kChains chains of DFMA on the first NF
 // lanes of each warp
 template <int KIND, int NF = 0, int NI = 0>
-__global__ void __launch_bounds__(256) k_rate(long long iters, double a, double b, double* out) {
+__global__ void __launch_bounds__(256) k_rate(long long iters, double a0, double b0, double* out) {
   if (KIND == 5 && (int)(threadIdx.x & 31) >= NF) return;
+  const double a = a0 - 1e-12 * threadIdx.x, b = b0 + 1e-15 * threadIdx.x;
   double x[kChains], z[NI > 0 ? NI : 1];
   float y[kChains];
 #pragma unroll
