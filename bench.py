@@ -45,17 +45,17 @@ ALG_BYTES_PER_CELL_UPDATE = 320  # stage 1: 64 B in + 64 B out; stage 2: 128 B i
 # DRAM traffic of one face-sweep launch (the x, y and z sweeps of a stage; mean of a stage-1 and a
 # stage-2 launch) from an ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum), valid only for the kernel sources it was taken on.
-TRAFFIC = {"face": {"bytes_per_launch": 1917.5e6, "cells": 160**3, "src": "684d1f6b83beb654"}}
+TRAFFIC = {"face": {"bytes_per_launch": 1917.3e6, "cells": 160**3, "src": "848cfdc0957518cb"}}
 # FP64 pipe slots (warp instructions) of the face sweep per 32 faces on the turbulence workload, mean of
 # a stage-1 and a stage-2 launch, from the same capture (sm__inst_executed_pipe_fp64). The kernel forms
 # part of the algorithm's operations on the integer and FP32 pipes, so its roofline is taken on the
 # slots it occupies of the pipe that bounds it; a slot counts as 2 flops, as in the measured peak.
-FP64_SLOTS = {"face": {"per_face": 102.4, "src": "684d1f6b83beb654"}}
+FP64_SLOTS = {"face": {"per_face": 102.4, "src": "848cfdc0957518cb"}}
 
 
 # what the face sweep's machine code is compiled from: its kernel, the numerics and indexing
 # headers, and the layout of the parameter struct it receives
-FACE_SOURCES = ("mhd_face.cu", "mhd_face.cuh", "mhd_device.cuh", "mhd_index.cuh")
+FACE_SOURCES = ("mhd_face.cu", "mhd_face.cuh", "mhd_device.cuh", "mhd_fixed.cuh", "mhd_index.cuh")
 
 
 def kernel_src_hash(files=FACE_SOURCES):
@@ -830,7 +830,8 @@ def main():
                                 "them run on the integer and FP32 pipes, so this can exceed the FP64 peak",
             "traffic": traffic,
             "peak_source": "FP64 measured on this GPU in this run: 2 flops x the DFMA rate of mhd_fp64_rate "
-                           "(independent chains on every SM)",
+                           "(independent chains on every SM, operands in registers; adds and multiplies reach "
+                           "0.84 of it, the face sweep's mix 0.89)",
             "frac_of_nominal": (slot_tflops if slot_tflops is not None else achieved) / FP64_PEAK_TFLOPS,
             "nominal_peak": FP64_PEAK_TFLOPS,
             "nominal_source": "152 SMs x 2 DFMA/clk x 2 flops x 2070 MHz (recipe SM count and maximum clock)",

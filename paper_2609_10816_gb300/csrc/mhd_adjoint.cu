@@ -3,15 +3,16 @@
 // The step is S1 = S0 + D(F(S0)), S2 = S0 + D((F(S0) + F(S1)) / 2), where F(S) collects the face
 // fluxes and edge EMFs of a state and D is the flux divergence / discrete curl (Eqs.
 // rk:increment-state, rk:increment-bfield). Reverse mode runs backwards through this chain; the
-// adjoint of F at a state is assembled from local Jacobians, each obtained with forward-mode
-// dual numbers on the GPU (one tangent per local input), so every limiter, min/max and
-// Riemann-fan branch is differentiated on the branch the forward pass took:
+// adjoint of F at a state is assembled from local reverse sweeps and Jacobians written by hand (the
+// face solve's is checked against forward-mode dual numbers by mhd_adjoint_check). Every limiter,
+// min/max and Riemann-fan branch is differentiated on the branch the forward pass took, decided on
+// values formed by the same functions and roundings:
 //   edges   : E = LD04(Q26 corners) from 8 reconstructed edge values and 4 edge speeds, + eta j
 //   edge rec: face fields and face velocities reconstructed to edges (point-wise reconstruction)
 //   faces   : Riemann solve from the 7 + 7 reconstructed states and the normal field
 //   face rec: primitives reconstructed to faces
 //   prim    : conserved variables and the face field to primitives
-// plus the Joule flux and eta j terms, which are bilinear and differentiated by hand. Adjoint
+// plus the Joule flux and eta j terms, which are bilinear. Adjoint
 // contributions that several threads add to the same face are accumulated with atomics.
 #include <cstring>
 #include <string>

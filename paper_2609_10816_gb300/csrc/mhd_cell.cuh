@@ -90,8 +90,9 @@ __device__ __forceinline__ double warp_max_leave(double s, double entered, unsig
 // not, and carry bounds of their own: p, the difference of energies, takes 2^-18 of e_tot more, and the
 // mean of two face values b, which may cancel (a field that alternates from face to face), lies within
 // 2^-23 (|lo| + |hi|) of its float, so that b^2 is taken at the upper end of that interval where it adds
-// to the speed and at the lower end where it takes from p. The FP64 instructions of a cell take 35 x 64 cycles of their pipe,
-// these about 100 of others: 192^3 turbulence, mhd_max_dt and mhd_divb 0.60 ms, so 0.32.
+// to the speed and at the lower end where it takes from p. The FP64 instructions of a cell take 35 x 64
+// cycles of their pipe, these about 120 of others: 192^3 turbulence, mhd_max_dt and mhd_divb 0.60 ms, so
+// 0.32.
 // Only states of ordinary size are judged (every value below 2^60, rho and e_tot positive and above
 // 2^-30, m above 2^-40, p certainly positive), so that nothing overflows, flushes to zero or is not a
 // number.

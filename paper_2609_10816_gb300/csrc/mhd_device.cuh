@@ -1,7 +1,7 @@
 // mhd_device.cuh -- device numerics of the CT-MHD step (FP64, sm_103a).
 //
-// On GB300 the FP64 pipe retires about 2 DFMA per SM per clock (measured ~0.59 T DFMA/s over
-// 152 SMs), 1/64 of the FP32 rate; a DMNMX or DSETP costs a full FP64 issue slot. Every
+// On GB300 the FP64 pipe retires 2 DFMA per SM per clock (measured 0.63 T DFMA/s over 152 SMs;
+// 0.53 T of adds or multiplies), 1/64 of the FP32 rate; a DMNMX or DSETP costs a full FP64 issue slot. Every
 // comparison, min/max, |x| and sign test below therefore runs on the integer pipe, on the
 // IEEE-754 bit pattern: for non-NaN doubles, the key  b ^ ((b >> 63) & 0x7fff...f)  of the bit
 // pattern b orders like the value (with -0 just below +0), and for non-negative values the raw
@@ -89,8 +89,9 @@ __device__ __forceinline__ bool finite_d(double x) {
 // 2^-32. Exponents at the ends of the range, zero, infinities and NaN take the hardware's FP64 seed
 // and one more term of the series, as does a negative argument of a root.
 // Measured (256^3 turbulence step): face sweeps 21.0 -> 19.5 ms, left/right edge sweeps 6.26 -> 5.91,
-// flag pass 1.17 -> 1.05; the 128^3 Alfven wave's face sweeps 4.67 -> 4.30. Largest errors over 10^8
-// hashed arguments, the seed's float off by up to 2 ulp either way: reciprocal 1.0, root 1.5 x 2^-53.
+// flag pass 1.17 -> 1.05; the 128^3 Alfven wave's face sweeps 4.67 -> 4.30. Largest differences from
+// IEEE results over 2^28 arguments of every binade (mhd_math_check): reciprocal and root 2.0, reciprocal
+// root 2.4 x 2^-53.
 __device__ __forceinline__ unsigned hi_word(double x) { return (unsigned)__double2hiint(x); }
 __device__ __forceinline__ double seed_bits(float f0, float c32, unsigned hi_scale) {
   // f0 + c32 2^-32, its exponent shifted by hi_scale (a multiple of 2^20 in the high word)
@@ -768,8 +769,8 @@ __device__ __noinline__ T fast_max_any(T rl, T rr, T Al, T Ar, bool& left) {
   return sqrt_(left ? cl : cr);
 }
 // The larger of the two fast speeds, sqrt(A / (2 rho)) of that side = (A/2) / sqrt(rho A/2): one
-// reciprocal square root in the place of two reciprocals and a square root (9 FP64 instructions
-// against 14).
+// reciprocal square root in the place of two reciprocals and a square root (7 FP64 instructions
+// against 9; 9 against 14 with the hardware's FP64 seeds).
 template <class T>
 __device__ __forceinline__ T fast_max(const FaceStateT<T>& sl, const FaceStateT<T>& sr, const PhysFluxT<T>& L,
                                       const PhysFluxT<T>& R) {
@@ -887,13 +888,13 @@ __device__ __forceinline__ FaceStateT<T> pick(bool left, const FaceStateT<T>& a,
 // (F + S (U* - U), and F* + S* (U** - U*)) the physical flux of the state at x/t = 0, with S_M for
 // its normal velocity and p_t* for its total pressure. So the branches only form that state
 // (density, tangential velocity and field, energy, u . b), and one flux is formed at the end by all
-// lanes of a warp together: in the fan 105 FP64 instructions a face against 143 when the flux
-// vectors were differenced across the waves, and 154 against 218 in the double-star region
-// (counted on the formulas; with fast_max and sqrt_ the 256^3 turbulence step took 46.9 ms against
-// 49.4, the 128^3 Alfven step 8.43 against 9.64, 96 subsonic patches 19.9 against 22.8). MK05
-// Eqs. 38 and 41 are taken relative to the side's own velocity:
-// d = S_M - u = (m_o (u_R - u_L) + p_L - p_R) / (m_R - m_L) with the other side's mass flux m_o,
-// and p_t* = p_t + m d.
+// lanes of a warp together: in the fan 90 FP64 instructions a face (speeds and flux, counted on the
+// formulas), in the double-star region 132; 105 and 154 with reciprocals of 3 instructions and roots of
+// 5, against 143 and 218 when the flux vectors were differenced across the waves (with fast_max and
+// sqrt_ the 256^3 turbulence step took 46.9 ms against 49.4, the 128^3 Alfven step 8.43 against 9.64,
+// 96 subsonic patches 19.9 against 22.8). MK05 Eqs. 38 and 41 are taken relative to the side's own
+// velocity: d = S_M - u = (m_o (u_R - u_L) + p_L - p_R) / (m_R - m_L) with the other side's mass flux
+// m_o, and p_t* = p_t + m d.
 // A component of the double-star state differs from the star state a of its side by
 // x = (sqrt(rho_b*) (v_b - v_a) + s (B_b - B_a)) / (sqrt(rho_a*) + sqrt(rho_b*)) in the velocity and
 // by s sqrt(rho_a*) x in the field (MK05 Eqs. 59-62, b the other side's star state, s = sgn(b_n)

@@ -16,9 +16,10 @@
 // and stores cover whole sectors.
 // Measured (face sweeps of a step; before / windows in registers, all unrolled; then as here with
 // the x sweep walked; by lanes): 256^3 turbulence PPM + HLLD 30.6, 22.8, 21.0 ms; 128^3 with the
-// FS18 EMF's extra stores 4.7, 3.9, 2.9 ms. With the two-instruction reciprocals 19.5 and 2.6: about
-// 110 FP64 warp instructions a face at 72 cycles each, which is what the pipe takes for mixed adds,
-// products and fused multiply-adds.
+// FS18 EMF's extra stores 4.7, 3.9, 2.9 ms. With the two-instruction reciprocals 19.5 and 2.6: 98 to
+// 107 FP64 warp instructions per 32 faces in 9.9 ms a launch at 256^3, about 77 cycles of their pipe
+// each, where a fused multiply-add alone takes 64, an add or a product 76, and this mix (a third fused)
+// 72.
 #pragma once
 #include "mhd_device.cuh"
 #include "mhd_index.cuh"

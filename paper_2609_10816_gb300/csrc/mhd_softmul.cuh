@@ -1,7 +1,7 @@
 // mhd_softmul.cuh -- binary64 multiply on the 32-bit integer pipe, for the FP64 rate probe and the
 // arithmetic self-check only.
 //
-// Every kernel of the step is bound by the FP64 pipe (about 1.6 results per SM per clock) while the
+// Every kernel of the step is bound by the FP64 pipe (1.7 to 2 results per SM per clock) while the
 // integer pipes stay mostly idle, so a product formed on the integer pipe would move work to the idle
 // unit. A product of two doubles is a short integer computation: the two 53-bit significands
 // multiply exactly in four 32 x 32 -> 64-bit multiply-adds, the 106-bit product is normalised by at
