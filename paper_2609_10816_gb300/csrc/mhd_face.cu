@@ -46,6 +46,16 @@ __global__ void __launch_bounds__(kFaceThreads, kFaceMinBlocks) k_faces(Dev D, i
 // that fills a lane sweep's windows (32^3, PLM + HLL: face sweeps of a step 114 us walked, 151 by
 // lanes; 64^3, PPM + HLLD, one stage with stored states: 388 against 384).
 constexpr long long kLaneCells = 1LL << 17;
+// Points per segment of a walked face sweep: fill_seg's, and less for boxes that leave the GPU idle,
+// though each segment starts its windows anew: a face in a walk waits for the one before it (about 7 us
+// each on an idle GPU; face sweeps of a PPM + HLLD step with 4, 2 and 1: 8^3 104, 67, 48 us; 24^3 108,
+// 88, 74; 32^3 144, 112, 128; 48^3 324, 292, 332).
+static int walk_seg(const Dev& d, int dir, int seg, long long resident_threads) {
+  int s = fill_seg(d, dir, seg, resident_threads);
+  if (s <= 4 && sweep_threads(d, dir, 2) <= resident_threads) s = 2;
+  if (s <= 2 && 3 * sweep_threads(d, dir, 1) <= resident_threads) s = 1;
+  return s;
+}
 template <int RC, int RS>
 static void launch_faces_t(const Dev& d, int seg, cudaStream_t st) {
   const int bs = kFaceThreads, smem = face_smem_bytes<RC>();
@@ -60,13 +70,7 @@ static void launch_faces_t(const Dev& d, int seg, cudaStream_t st) {
       while (sg[dir] > 8 && lane_threads(d, dir, sg[dir]) < 2 * res * bs) sg[dir] = lane_seg(sg[dir] / 2);
       tot += lane_threads(d, dir, sg[dir]);
     } else {
-      sg[dir] = fill_seg(d, dir, seg, res * bs);
-      // a face in a walk waits for the one before it (about 7 us each on an idle GPU), so boxes that
-      // leave it idle walk 2 faces, and the smallest one, though each walk starts its windows anew
-      // (face sweeps of a PPM + HLLD step with 4, 2 and 1: 8^3 104, 67, 48 us; 24^3 108, 88, 74;
-      // 32^3 144, 112, 128; 48^3 324, 292, 332)
-      if (sg[dir] <= 4 && sweep_threads(d, dir, 2) <= res * bs) sg[dir] = 2;
-      if (sg[dir] <= 2 && 3 * sweep_threads(d, dir, 1) <= res * bs) sg[dir] = 1;
+      sg[dir] = walk_seg(d, dir, seg, res * bs);
       tot += sweep_threads(d, dir, sg[dir]) + 31;
     }
   }
@@ -77,9 +81,13 @@ static void launch_faces_t(const Dev& d, int seg, cudaStream_t st) {
 template <int RC, int RS>
 static void launch_face_t(const Dev& d, int dir, int seg, cudaStream_t st) {
   const int bs = kFaceThreads, smem = face_smem_bytes<RC>();
-  const long long threads = sweep_threads(d, dir, seg);
-  resident_blocks((const void*)k_face<RC, RS>, bs, smem);  // (allows the kernel its shared memory)
-  k_face<RC, RS><<<(unsigned)((threads + bs - 1) / bs), bs, smem, st>>>(d, dir, seg);
+  // (the call also allows the kernel its shared memory. Segments of 64 faces whatever the box left its
+  // chains of steps too long: mhd_step_noalloc at 32^3, PC + LLF 1.59 ms, so 0.47; PPM + HLLD 0.78, 4.03
+  // with the windows in registers)
+  const long long res = resident_blocks((const void*)k_face<RC, RS>, bs, smem);
+  const int sg = walk_seg(d, dir, seg, res * bs);
+  const long long threads = sweep_threads(d, dir, sg);
+  k_face<RC, RS><<<(unsigned)((threads + bs - 1) / bs), bs, smem, st>>>(d, dir, sg);
 }
 
 template <int RC>
