@@ -249,10 +249,13 @@ __device__ __forceinline__ void face_thread(const Dev& D, int dir, bool by_lanes
 }
 
 // Whether the sweep along dir runs as a lane sweep: along x, on lines of at least 16 points with at
-// most a sixteenth of the lanes idle in a line's last pass.
+// most a sixteenth of the lanes idle in a line's last pass, and of those in the last group of 4 lines
+// (2^22 cells, PPM + HLLD step, by lanes and walked: 1 line 20.2 and 13.2 ms, 2 lines 16.1 and 13.7, 5
+// lines 14.1 and 12.8, 13 lines 13.2 and 13.1, 26 lines 13.7 and 14.0, 64 x 64 lines 11.9 and 12.4).
 __host__ __device__ __forceinline__ bool face_by_lanes(const Dev& D, int dir) {
   const int n = D.n[dir];
-  return dir == 0 && n >= 16 && (n + 7) / 8 * 120 <= 16 * n;
+  const long long lines = (long long)D.n[1] * D.n[2];
+  return dir == 0 && n >= 16 && (n + 7) / 8 * 120LL <= 16LL * n && (lines + 3) / 4 * 60 <= 16 * lines;
 }
 
 }  // namespace mhd
