@@ -45,12 +45,12 @@ ALG_BYTES_PER_CELL_UPDATE = 320  # stage 1: 64 B in + 64 B out; stage 2: 128 B i
 # DRAM traffic of one face-sweep launch (the x, y and z sweeps of a stage; mean of a stage-1 and a
 # stage-2 launch) from an ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum), valid only for the kernel sources it was taken on.
-TRAFFIC = {"face": {"bytes_per_launch": 1917.3e6, "cells": 160**3, "src": "848cfdc0957518cb"}}
+TRAFFIC = {"face": {"bytes_per_launch": 1917.7e6, "cells": 160**3, "src": "b1f91f2f38c9a69e"}}
 # FP64 pipe slots (warp instructions) of the face sweep per 32 faces on the turbulence workload, mean of
 # a stage-1 and a stage-2 launch, from the same capture (sm__inst_executed_pipe_fp64). The kernel forms
 # part of the algorithm's operations on the integer and FP32 pipes, so its roofline is taken on the
 # slots it occupies of the pipe that bounds it; a slot counts as 2 flops, as in the measured peak.
-FP64_SLOTS = {"face": {"per_face": 102.4, "src": "848cfdc0957518cb"}}
+FP64_SLOTS = {"face": {"per_face": 102.4, "src": "b1f91f2f38c9a69e"}}
 
 
 # what the face sweep's machine code is compiled from: its kernel, the numerics and indexing
